@@ -116,7 +116,8 @@ void fill_table_image(const mpf_profile *p, const TableGeom &g, int fmt, uint8_t
   };
   auto put = [&](size_t off, int x, int k) {
     const int sv = score(x, k);
-    const uint16_t bits = fmt == TABLE_F16 ? half_bits(sv) : (uint16_t)(int16_t)sv;
+    const uint16_t bits = fmt == TABLE_F16 ? half_bits(sv)
+                                           : (uint16_t)(int16_t)(sv == kNegInf ? kNegInf : sv * (1 << kCellShift));
     memcpy(&img[off], &bits, 2);
   };
   const int qw = 4 * g.quads;   // words held in the quad region
@@ -845,6 +846,7 @@ int enqueue_group(const mpf_db *db, mpf_ctx *ctx, LaunchGroup &g, cudaStream_t s
   sp.tile_col_stride = g.col_stride;
   sp.tile_col_bytes = g.col_bytes;
   sp.qp_table_stride = g.qp_stride;
+  sp.one = 1;
   const uint64_t n_items = ((uint64_t)g.n_queries + (uint64_t)g.qp - 1) / (uint64_t)g.qp * g.n_shards;
   const int grid = (int)std::min<uint64_t>((uint64_t)g.grid, n_items);
   g.fn<<<grid, g.threads, g.smem, st>>>(sp);

@@ -32,7 +32,17 @@ __device__ __forceinline__ uint32_t dynamic_smem_bytes() {
 // row leaves every score unchanged (the paper's '#' residue, Sec. 3.2).
 constexpr int kPadCode = 32;
 constexpr int kTableRows = 33;           // codes 0..31 plus padding
-constexpr int kNegInf = -16384;          // score of padding rows and nodes > M
+constexpr int kNegInf = -16384;          // table entry of padding rows and nodes > M
+// Integer cells and table entries of the striped kernels hold scores in units
+// of 2^kCellShift (every score and cell that counts is below 510 in
+// magnitude, so 16 bits hold it).  The low bits take the carries that 32-bit
+// sums of packed cells leave in the upper half: at most one per pair of
+// rows, cleared every kClearSteps steps of four rows, before they reach a
+// unit.
+constexpr int kCellShift = 6;
+constexpr int kClearSteps = 30;
+constexpr uint32_t kCellMask2 = 0xffc0ffc0u;
+static_assert(2 * kClearSteps < (1 << kCellShift), "carries stay below one score unit");
 constexpr int kBlockThreads = 512;
 constexpr int kMaxWords = 48;
 constexpr int kStripedMaxM = 2 * 32 * kMaxWords;   // longest model of the striped kernels
@@ -130,6 +140,7 @@ struct ScanParams {
   uint8_t *tile_col;          // tiled kernel: per resident warp two columns of
   uint32_t tile_col_stride;   //   tile_col_stride bytes (an int16 per row)
   uint64_t tile_col_bytes;
+  uint32_t one;               // 1 (striped kernels: see add_imad)
   uint32_t qp_table_stride;   // striped kernels with several queries per warp: bytes per staged table
 };
 

@@ -121,6 +121,7 @@ extern "C" int mpf_scan_noalloc(mpf_ctx *ctx, int filter, const mpf_profile *pro
   MPF_CUDA(cudaMemsetAsync(scratch + 256, 0, 4, ctx->stream));
 
   ScanParams sp{};
+  sp.one = 1;
   sp.residues = db->d_words;
   sp.n_words = db->n_words;
   sp.seq_word = db->d_seq_word;
