@@ -50,6 +50,16 @@ KernelFn kernel_qp_tm(int lanes, int words, int mode) {
     default: return nullptr;
   }
 }
+KernelFn kernel_qp_tmfew(int lanes, int words, int mode) {
+  switch (lanes) {
+    case 1: return kernel_qp_tmfew_lg1(words, mode);
+    case 2: return kernel_qp_tmfew_lg2(words, mode);
+    case 4: return kernel_qp_tmfew_lg4(words, mode);
+    case 8: return kernel_qp_tmfew_lg8(words, mode);
+    case 16: return kernel_qp_tmfew_lg16(words, mode);
+    default: return nullptr;
+  }
+}
 }  // namespace mpf
 
 // ---------------------------------------------------------------- helpers --
@@ -360,6 +370,7 @@ struct LaunchGroup {
   int threads = kBlockThreads;
   uint32_t long_words = 0;       // long-model kernel: largest seg_words of the group
   int n_codes = 32;              // distinct residue codes of the database
+  uint32_t tm_rows = kTableRows; // its largest code + 1, and one (rows of a few-codes TMEM table)
   uint32_t n_shards = 0;
   QueryDesc *d_queries = nullptr;
   uint32_t n_queries = 0;
@@ -483,9 +494,15 @@ int configure_kernel(mpf_ctx *ctx, LaunchGroup *g) {
     g->n_shards = (uint32_t)g->grid;
     return MPF_OK;
   }
-  g->fn = g->qp > 1 ? kernel_qp_tm(g->lanes, g->words, g->mode)
-         : g->tm    ? kernel_lg32_tm(g->words, g->mode)
-                    : kernel_for(g->lanes, g->words, g->mode);
+  // With the table in tensor memory: the few-codes kernel where the
+  // database's codes allow it and it is built.
+  g->fn = nullptr;
+  if (g->tm && g->tm_rows <= kTmFewCodes + 1)
+    g->fn = g->qp > 1 ? kernel_qp_tmfew(g->lanes, g->words, g->mode) : kernel_lg32_tmfew(g->words, g->mode);
+  if (!g->fn)
+    g->fn = g->qp > 1 ? kernel_qp_tm(g->lanes, g->words, g->mode)
+           : g->tm    ? kernel_lg32_tm(g->words, g->mode)
+                      : kernel_for(g->lanes, g->words, g->mode);
   if (!g->fn) return MPF_EINVAL;
   g->smem = g->qp > 1 ? (uint32_t)g->qp * g->qp_stride : (uint32_t)smem_need(g->lanes, g->words);
   if (g->smem > (uint32_t)ctx->max_smem) return MPF_EUNSUPPORTED;
@@ -497,7 +514,7 @@ int configure_kernel(mpf_ctx *ctx, LaunchGroup *g) {
                                 (int)g->smem));
   int per_sm = 0;
   MPF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)g->fn,
-                                                         kBlockThreads, g->smem));
+                                                         g->threads, g->smem));
   if (per_sm < 1 || (g->tm && per_sm != 1)) return MPF_EUNSUPPORTED;
   g->grid = ctx->num_sms * per_sm;
   g->n_shards = (uint32_t)g->grid * (uint32_t)std::max(1, g->shard_factor);
@@ -728,6 +745,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     g.shard_factor = group_shards[kv.first];
     for (const QueryDesc &qd : kv.second) g.long_words = std::max(g.long_words, qd.seg_words);
     g.n_codes = db->n_codes;
+    g.tm_rows = (uint32_t)db->code_end + 1u;
     int rc = configure_kernel(ctx, &g);
     if (rc) {
       plan_free(pl);
@@ -847,6 +865,7 @@ int enqueue_group(const mpf_db *db, mpf_ctx *ctx, LaunchGroup &g, cudaStream_t s
   sp.tile_col_bytes = g.col_bytes;
   sp.qp_table_stride = g.qp_stride;
   sp.one = 1;
+  sp.tm_rows = g.tm_rows;
   const uint64_t n_items = ((uint64_t)g.n_queries + (uint64_t)g.qp - 1) / (uint64_t)g.qp * g.n_shards;
   const int grid = (int)std::min<uint64_t>((uint64_t)g.grid, n_items);
   g.fn<<<grid, g.threads, g.smem, st>>>(sp);
@@ -1244,6 +1263,7 @@ int mpf_db_upload(mpf_ctx *ctx, const uint8_t *residues, uint64_t n_residues,
   for (uint64_t s = 0; s < n_seqs; ++s) db->n_residues += lengths[s];
   db->pad_word = 0;
   db->n_codes = __builtin_popcount(seen);
+  db->code_end = seen ? 32 - __builtin_clz(seen) : 1;
   db->max_len = n_seqs ? seq_len[0] : 0;
   const size_t ns = std::max<uint64_t>(n_seqs, 1);
   db->n_words = (uint32_t)(chunks * 4);

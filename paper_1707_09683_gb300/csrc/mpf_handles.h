@@ -71,6 +71,7 @@ struct mpf_db {
   uint32_t *d_seq_orig = nullptr;
   uint32_t pad_word = 0;
   int n_codes = 0;                  // distinct residue codes present
+  int code_end = 32;                // largest residue code present + 1
   uint32_t max_len = 0;             // longest sequence
 };
 

@@ -8,6 +8,9 @@
 // words).  With -DMPF_QP=1 (lanes 1 to 16) it builds kernel_qp_tm_lg<lanes>():
 // the tensor-memory variants that score one sequence against 32 / lanes
 // queries per warp (integer SSV, the held MSV pass and the two together).
+// Either with -DMPF_FEW=1 builds the variants for databases of few residue
+// codes (kernel_lg32_tmfew(), kernel_qp_tmfew_lg<lanes>(): those three modes,
+// from 16 words on; shorter lanes fit tensor memory whole with every code).
 #include "mpf_scan_kernel.cuh"
 
 #ifndef MPF_LG
@@ -16,40 +19,47 @@
 #define MPF_CAT2(a, b) a##b
 #define MPF_CAT(a, b) MPF_CAT2(a, b)
 
+// C(words) for each word count of a range.
+#define MPF_WORDS_4_6(C) C(4) C(6)
+#define MPF_WORDS_8_14(C) C(8) C(10) C(12) C(14)
+#define MPF_WORDS_16_48(C)                                                                \
+  C(16) C(18) C(20) C(22) C(24) C(26) C(28) C(30) C(32) C(34) C(36) C(38) C(40) C(42)     \
+  C(44) C(46) C(48)
+
 namespace mpf {
 
-#if defined(MPF_QP)
+#if defined(MPF_QP) || (defined(MPF_TM) && defined(MPF_FEW))
 
-#define MPF_WORDS_CASE(W)                                                                             \
-  case W:                                                                                             \
-    if (mode == MODE_SSV) return scan_kernel<MPF_LG, W, MODE_SSV, true, 32 / MPF_LG>;                 \
-    if (mode == MODE_MSV_HELD) return scan_kernel<MPF_LG, W, MODE_MSV_HELD, true, 32 / MPF_LG>;       \
-    if (mode == MODE_MSV_SSV) return scan_kernel<MPF_LG, W, MODE_MSV_SSV, true, 32 / MPF_LG>;         \
+#ifdef MPF_QP
+constexpr int kQueries = 32 / MPF_LG;
+#else
+constexpr int kQueries = 1;
+#endif
+#ifdef MPF_FEW
+constexpr int kTable = TM_FEW;
+#else
+constexpr int kTable = TM_ALL;
+#endif
+
+#define MPF_CASE(W)                                                                           \
+  case W:                                                                                     \
+    if (mode == MODE_SSV) return scan_kernel<MPF_LG, W, MODE_SSV, kTable, kQueries>;          \
+    if (mode == MODE_MSV_HELD) return scan_kernel<MPF_LG, W, MODE_MSV_HELD, kTable, kQueries>; \
+    if (mode == MODE_MSV_SSV) return scan_kernel<MPF_LG, W, MODE_MSV_SSV, kTable, kQueries>;  \
     return nullptr;
 
+#if defined(MPF_QP) && defined(MPF_FEW)
+KernelFn MPF_CAT(kernel_qp_tmfew_lg, MPF_LG)(int words, int mode) {
+#elif defined(MPF_QP)
 KernelFn MPF_CAT(kernel_qp_tm_lg, MPF_LG)(int words, int mode) {
+#else
+KernelFn kernel_lg32_tmfew(int words, int mode) {
+#endif
   switch (words) {
-    MPF_WORDS_CASE(8)
-    MPF_WORDS_CASE(10)
-    MPF_WORDS_CASE(12)
-    MPF_WORDS_CASE(14)
-    MPF_WORDS_CASE(16)
-    MPF_WORDS_CASE(18)
-    MPF_WORDS_CASE(20)
-    MPF_WORDS_CASE(22)
-    MPF_WORDS_CASE(24)
-    MPF_WORDS_CASE(26)
-    MPF_WORDS_CASE(28)
-    MPF_WORDS_CASE(30)
-    MPF_WORDS_CASE(32)
-    MPF_WORDS_CASE(34)
-    MPF_WORDS_CASE(36)
-    MPF_WORDS_CASE(38)
-    MPF_WORDS_CASE(40)
-    MPF_WORDS_CASE(42)
-    MPF_WORDS_CASE(44)
-    MPF_WORDS_CASE(46)
-    MPF_WORDS_CASE(48)
+#ifndef MPF_FEW
+    MPF_WORDS_8_14(MPF_CASE)
+#endif
+    MPF_WORDS_16_48(MPF_CASE)
     default:
       return nullptr;
   }
@@ -57,40 +67,21 @@ KernelFn MPF_CAT(kernel_qp_tm_lg, MPF_LG)(int words, int mode) {
 
 #elif defined(MPF_TM) && MPF_LG == 32
 
-#define MPF_WORDS_CASE(W)                                                                  \
-  case W:                                                                                  \
-    if (mode == MODE_SSV) return scan_kernel<32, W, MODE_SSV, true>;                       \
-    if (mode == MODE_MSV_FAST) return scan_kernel<32, W, MODE_MSV_FAST, true>;             \
-    if (mode == MODE_SSV_F16) return scan_kernel<32, W, MODE_SSV_F16, true>;               \
-    if (mode == MODE_MSV_FAST_F16) return scan_kernel<32, W, MODE_MSV_FAST_F16, true>;     \
-    if (mode == MODE_MSV_HELD) return scan_kernel<32, W, MODE_MSV_HELD, true>;             \
-    if (mode == MODE_MSV_HELD_F16) return scan_kernel<32, W, MODE_MSV_HELD_F16, true>;     \
-    if (mode == MODE_MSV_SSV) return scan_kernel<32, W, MODE_MSV_SSV, true>;               \
+#define MPF_CASE(W)                                                                      \
+  case W:                                                                                \
+    if (mode == MODE_SSV) return scan_kernel<32, W, MODE_SSV, TM_ALL>;                   \
+    if (mode == MODE_MSV_FAST) return scan_kernel<32, W, MODE_MSV_FAST, TM_ALL>;         \
+    if (mode == MODE_SSV_F16) return scan_kernel<32, W, MODE_SSV_F16, TM_ALL>;           \
+    if (mode == MODE_MSV_FAST_F16) return scan_kernel<32, W, MODE_MSV_FAST_F16, TM_ALL>; \
+    if (mode == MODE_MSV_HELD) return scan_kernel<32, W, MODE_MSV_HELD, TM_ALL>;         \
+    if (mode == MODE_MSV_HELD_F16) return scan_kernel<32, W, MODE_MSV_HELD_F16, TM_ALL>; \
+    if (mode == MODE_MSV_SSV) return scan_kernel<32, W, MODE_MSV_SSV, TM_ALL>;           \
     return nullptr;
 
 KernelFn kernel_lg32_tm(int words, int mode) {
   switch (words) {
-    MPF_WORDS_CASE(8)
-    MPF_WORDS_CASE(10)
-    MPF_WORDS_CASE(12)
-    MPF_WORDS_CASE(14)
-    MPF_WORDS_CASE(16)
-    MPF_WORDS_CASE(18)
-    MPF_WORDS_CASE(20)
-    MPF_WORDS_CASE(22)
-    MPF_WORDS_CASE(24)
-    MPF_WORDS_CASE(26)
-    MPF_WORDS_CASE(28)
-    MPF_WORDS_CASE(30)
-    MPF_WORDS_CASE(32)
-    MPF_WORDS_CASE(34)
-    MPF_WORDS_CASE(36)
-    MPF_WORDS_CASE(38)
-    MPF_WORDS_CASE(40)
-    MPF_WORDS_CASE(42)
-    MPF_WORDS_CASE(44)
-    MPF_WORDS_CASE(46)
-    MPF_WORDS_CASE(48)
+    MPF_WORDS_8_14(MPF_CASE)
+    MPF_WORDS_16_48(MPF_CASE)
     default:
       return nullptr;
   }
@@ -98,7 +89,7 @@ KernelFn kernel_lg32_tm(int words, int mode) {
 
 #else
 
-#define MPF_WORDS_CASE(W)                                                            \
+#define MPF_CASE(W)                                                                  \
   case W:                                                                            \
     if (mode == MODE_SSV) return scan_kernel<MPF_LG, W, MODE_SSV>;                   \
     if (mode == MODE_MSV_FAST) return scan_kernel<MPF_LG, W, MODE_MSV_FAST>;         \
@@ -112,29 +103,9 @@ KernelFn kernel_lg32_tm(int words, int mode) {
 
 KernelFn MPF_CAT(kernel_lg, MPF_LG)(int words, int mode) {
   switch (words) {
-    MPF_WORDS_CASE(4)
-    MPF_WORDS_CASE(6)
-    MPF_WORDS_CASE(8)
-    MPF_WORDS_CASE(10)
-    MPF_WORDS_CASE(12)
-    MPF_WORDS_CASE(14)
-    MPF_WORDS_CASE(16)
-    MPF_WORDS_CASE(18)
-    MPF_WORDS_CASE(20)
-    MPF_WORDS_CASE(22)
-    MPF_WORDS_CASE(24)
-    MPF_WORDS_CASE(26)
-    MPF_WORDS_CASE(28)
-    MPF_WORDS_CASE(30)
-    MPF_WORDS_CASE(32)
-    MPF_WORDS_CASE(34)
-    MPF_WORDS_CASE(36)
-    MPF_WORDS_CASE(38)
-    MPF_WORDS_CASE(40)
-    MPF_WORDS_CASE(42)
-    MPF_WORDS_CASE(44)
-    MPF_WORDS_CASE(46)
-    MPF_WORDS_CASE(48)
+    MPF_WORDS_4_6(MPF_CASE)
+    MPF_WORDS_8_14(MPF_CASE)
+    MPF_WORDS_16_48(MPF_CASE)
     default:
       return nullptr;
   }

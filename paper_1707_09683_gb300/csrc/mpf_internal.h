@@ -71,17 +71,19 @@ enum Mode : int {
 constexpr int kNumModes = 8;   // modes of the striped scan kernel
 
 // Striped kernels that read their table from tensor memory (one sequence per
-// warp): the first tm_words(words) words of each lane's row of every residue
-// code (all 33 rows: 33 x 14 = 462 of the 512 columns) come from TMEM, the
-// rest from shared memory.
+// warp): the first words of each lane's row of every residue code come from
+// TMEM, the rest from shared memory.  A database whose codes are all below
+// kTmFewCodes needs few rows (its codes and the padding code), so 24 words of
+// each fit the 512 columns (21 x 24 = 504); otherwise all 33 rows are held,
+// with 12 words, or all of up to 14 (33 x 14 = 462).
 constexpr uint32_t kTmemColumns = 512;   // 32-bit columns of an SM's tensor memory
-constexpr int kTmWordsAll = 14;     // lanes of up to this many words: all of them in TMEM
-constexpr int kTmWordsPart = 12;    // longer lanes: this many in TMEM (a whole number of chunks)
 constexpr int kTmMinWords = 8;      // fewer words per lane: the shared-memory kernels
-// Words per lane read from TMEM for a lane of `words` words.  Twelve words
-// take the shared-memory reads of a 48-word lane to 3/4 of the table, below
-// the rate at which the integer pipe can use them.
-__host__ __device__ constexpr int tm_words(int words) { return words <= kTmWordsAll ? words : kTmWordsPart; }
+constexpr int kTmFewCodes = 20;
+enum TmTable : int { TM_NONE = 0, TM_ALL = 1, TM_FEW = 2 };   // table in shared memory; TMEM, all codes; TMEM, few codes
+// Words per lane read from TMEM for a lane of `words` words.
+__host__ __device__ constexpr int tm_words(int words, int tm) {
+  return tm == TM_NONE ? 0 : tm == TM_FEW ? (words <= 24 ? words : 24) : (words <= 14 ? words : 12);
+}
 
 // Score-table formats: signed 16-bit integers, or the same integers as fp16.
 // TABLE_I16_PACKED: integer scores in the packed geometry (one copy of each
@@ -140,6 +142,7 @@ struct ScanParams {
   uint8_t *tile_col;          // tiled kernel: per resident warp two columns of
   uint32_t tile_col_stride;   //   tile_col_stride bytes (an int16 per row)
   uint64_t tile_col_bytes;
+  uint32_t tm_rows;           // TM_FEW kernels: TMEM rows, the database's codes and the padding code
   uint32_t one;               // 1 (striped kernels: see add_imad)
   uint32_t qp_table_stride;   // striped kernels with several queries per warp: bytes per staged table
 };
@@ -253,11 +256,20 @@ int viterbi_shape_key(bool fast, int Mpad, int n_codes, int max_smem, int num_sm
 
 // Kernel instantiation for (lanes, words, mode), or nullptr if not built.
 KernelFn kernel_for(int lanes, int words, int mode);
-// The tensor-memory variant (lanes = 32), or nullptr if not built.
+// The tensor-memory variants (lanes = 32) for databases of any codes and of
+// few (TM_FEW: the integer SSV, held MSV and one-sweep modes, from the word
+// counts on where it differs), or nullptr if not built.
 KernelFn kernel_lg32_tm(int words, int mode);
+KernelFn kernel_lg32_tmfew(int words, int mode);
 // Tensor-memory variants that score one sequence against 32 / lanes queries
 // per warp (lanes 1 to 16), or nullptr if not built.
 KernelFn kernel_qp_tm(int lanes, int words, int mode);
+KernelFn kernel_qp_tmfew(int lanes, int words, int mode);
+KernelFn kernel_qp_tmfew_lg1(int words, int mode);
+KernelFn kernel_qp_tmfew_lg2(int words, int mode);
+KernelFn kernel_qp_tmfew_lg4(int words, int mode);
+KernelFn kernel_qp_tmfew_lg8(int words, int mode);
+KernelFn kernel_qp_tmfew_lg16(int words, int mode);
 KernelFn kernel_qp_tm_lg1(int words, int mode);
 KernelFn kernel_qp_tm_lg2(int words, int mode);
 KernelFn kernel_qp_tm_lg4(int words, int mode);

@@ -63,13 +63,20 @@
 //
 // Tensor-memory variant (TM, one sequence per warp, LG = 32).  The table is
 // staged in shared memory as usual; then the first HT words of each lane's
-// row (all H up to 14 words, else 12) of all 33 residue rows are copied into
-// the block's tensor memory (thread t of warp w owns TMEM lane 32 (w mod 4) +
-// t: its row of code x is columns x * HT .. x * HT + HT - 1).  The TMEM loads
-// of a row are issued while the previous row is computed; the row then
-// updates its words past HT from shared memory and its first HT words from
-// the loaded registers.  Every row takes the same path, so the kernel has no
-// per-row branch on the table source.  The cell arithmetic is unchanged.
+// row are copied into the block's tensor memory (thread t of warp w owns TMEM
+// lane 32 (w mod 4) + t: its row of code x is columns x * HT .. x * HT + HT -
+// 1), for all 33 residue rows (TM_ALL: all H words up to 14, else 12) or, when
+// every code of the database is below 20, for those codes and the padding
+// code (TM_FEW: 24 words).  The kernel was held by shared memory's 128 B per
+// clock for the words past HT: of a lane's 38 words (M = 2405) 26 came from
+// there, 14 do with TM_FEW, and up to 24 words (M = 1536) none.  A row updates
+// its words past HT from shared memory, then its TMEM words from the highest
+// down; they come in two loads, each issued half a row ahead, so that a lane
+// holds one row's TMEM words and not two (24 words in two buffers would not
+// leave room for the cells).  Every row takes the same path, so the kernel
+// has no per-row branch on the table source.  Measured (GB300, 60,000
+// sequences, SSV, GCUPS): M = 2405 22,790 with TM_ALL, 25,140 with TM_FEW; 16
+// queries of M = 100 packed 23,950.  ncu at M = 2405: ALU pipe 67% -> 75%.
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -153,13 +160,13 @@ __device__ __forceinline__ uint32_t pack2_half(int v) {
   return (h << 16) | h;
 }
 
-template <int LG, int H, int MODE, bool TM = false, int QP = 1>
+template <int LG, int H, int MODE, int TM = TM_NONE, int QP = 1>
 __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   static_assert((H % 4 == 0 || H % 4 == 2) && H >= 4 && H <= kMaxWords, "words per lane");
   static_assert(!TM || ((LG == 32 || QP * LG == 32) && H >= kTmMinWords && MODE != MODE_MSV_DIRECT),
                 "tensor-memory variant");
   static_assert(QP == 1 || (TM && QP * LG == 32), "queries per warp");
-  constexpr int HT = TM ? tm_words(H) : 0;   // words per lane from TMEM
+  constexpr int HT = tm_words(H, TM);   // words per lane from TMEM
   static_assert(HT == H || HT % 4 == 0, "shared-memory words start on a chunk");
   constexpr int Q = H / 4;               // full 4-word chunks per lane and row
   constexpr bool kTail = (H % 4) == 2;   // two more words from the tail region
@@ -193,6 +200,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   // QP > 1: the 32 / LG groups of a warp score one sequence against QP
   // queries (the QP consecutive queries of a work item), so every lane of
   // the warp reads the same residue and the TMEM column of a row is uniform.
+  // Every lane of a warp follows the same sequence: a warp reduction (whose
+  // result is uniform) hands each residue word to the rows.
+  constexpr bool kUniform = TM != TM_NONE;
   const uint32_t n_items = (p.n_queries + QP - 1) / QP * p.n_shards;
   const int warp = (int)(threadIdx.x >> 5);
   uint32_t tm_lane = 0;   // TMEM address of this warp's lane quarter, column 0
@@ -203,6 +213,8 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
     tm_fence_after();
     tm_lane = s_tmem + ((uint32_t)((warp & 3) * 32) << 16);
   }
+  // TMEM rows: codes 0 .. tm_pad - 1, then the padding code.
+  const uint32_t tm_pad = TM == TM_FEW ? p.tm_rows - 1u : (uint32_t)kTableRows - 1u;
 
   for (;;) {
     if (threadIdx.x == 0) {
@@ -261,8 +273,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       // staged table into tensor memory: warp q < 4 writes lane quarter q.
       tm_fence_after();
       if (warp < 4) {
-        for (uint32_t x = 0; x < (uint32_t)kTableRows; ++x) {
-          const uint32_t col = tm_lane + x * (uint32_t)HT;
+        for (uint32_t row = 0; row <= tm_pad; ++row) {
+          const uint32_t col = tm_lane + row * (uint32_t)HT;
+          const uint32_t x = row == tm_pad ? (uint32_t)kPadCode : row;
 #pragma unroll
           for (int j = 0; j < HT / 4; ++j) {
             const uint4 s4 = *reinterpret_cast<const uint4 *>(tbl_lane + x * qd->row_bytes + j * LG * 16);
@@ -344,26 +357,25 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       for (int q = 0; q < H; ++q) v[q] = 0u;
       uint32_t vacc = 0u;
       uint32_t cur = __ldg(p.residues + (nsteps > 0 ? wptr : p.pad_word));
+      if constexpr (kUniform) cur = __reduce_max_sync(kFull, cur);
+      // The residue word after cur, as loaded.
+      uint32_t ahead = __ldg(p.residues + (1 < nsteps ? wptr + 1u : p.pad_word));
 
-      // Tensor-memory words of the current and the next row: the loads of
-      // row i + 1 are issued while row i is computed.  Every residue code,
-      // the padding code included, has a TMEM row (code x: columns x * HT ..).
-      // Whole-warp kernels of up to 16 words per lane: one 16-column load per
-      // row (tcgen05.ld .x16, one uniform address) in place of two or three
-      // narrower ones; the columns past a code's HT words belong to the next
-      // code (or lie past the 33 codes, inside the allocation) and are not
-      // used.  Measured per row of M = 600-1000: 3.5-8.5% faster; from 22
-      // words on, where a row has more work to hide the loads behind, the
-      // exact-width loads were up to 2% faster.  Packed kernels load HT
-      // columns (their group state leaves no registers for wider buffers).
-      constexpr int HL = TM ? ((QP == 1 && H <= 16) ? 16 : HT) : 1;
-      static_assert(!TM || (HT <= 16 && (kTableRows - 1) * HT + 16 <= (int)kTmemColumns), "load width");
-      uint32_t TA[HL], TB[HL];
+      // Tensor-memory words of a row come in two loads, the low words and the
+      // high words (processed first, after the words in shared memory); each
+      // load is issued while the row before its use is half done, so a lane
+      // holds one row's words and not two.  Either load may bring columns of
+      // the same row past those it is for; they are not used.
+      constexpr int HI = TM == TM_NONE ? 0 : HT <= 12 ? 4 : 8;
+      constexpr int LO = HT - HI;
+      constexpr int LOW = TM == TM_NONE ? 1 : LO <= 4 ? 4 : LO <= 8 ? 8 : 16;
+      static_assert(TM == TM_NONE || (LO >= 4 && LOW <= HT && LO <= 16), "load widths");
+      uint32_t tlo[LOW], thi[HI > 0 ? HI : 1];
       auto tm_col = [&](uint32_t xc) -> uint32_t {
         if (!MPF_DCHECK(p.status, xc < (uint32_t)kTableRows)) xc = kPadCode;
-        return tm_lane + xc * (uint32_t)HT;
+        return tm_lane + (TM == TM_FEW ? min(xc, tm_pad) : xc) * (uint32_t)HT;
       };
-      if constexpr (TM) tm_ld<HL>(TA, tm_col(cur & 0xffu));   // first row of the sequence
+      if constexpr (TM) tm_ld_pow2<HI>(thi, tm_col(cur & 0xffu) + LO);   // first row of the sequence
 
       // Four rows of one residue word (nxt: the next word).  CHECK: test every
       // row for the MSV threshold (only needed when some lane is near it, or
@@ -372,17 +384,15 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         constexpr bool CHECK = decltype(check_tag)::value;
 #pragma unroll
         for (int rr = 0; rr < 4; ++rr) {
-         auto one_row = [&](auto &Tc, auto &Tn) {
+         {
           // Rows past the end of a sequence read padding codes: their cells
           // score kNegInf, and the special states must not see them.
           const bool real = active && (4 * step + rr) < len;
           uint32_t x = __byte_perm(cur, 0u, 0x4440u + rr);   // residue code of row rr
           if (!MPF_DCHECK(p.status, x < (uint32_t)kTableRows)) x = kPadCode;
           if constexpr (TM) {
-            // This row's TMEM words (issued one row earlier), then the next
-            // row's loads: a wait covers every earlier load of the thread.
-            tm_wait_ld<HL>(Tc);
-            tm_ld<HL>(Tn, tm_col(rr < 3 ? __byte_perm(cur, 0u, 0x4440u + rr + 1) : nxt & 0xffu));
+            tm_wait_ld<HI>(thi);
+            tm_ld_pow2<LOW>(tlo, tm_col(x));
           }
           const uint8_t *rowp = tbl_lane + x * row_bytes;
           // Diagonal shift (Alg. 5): cell k-1 of the previous row feeds cell k.
@@ -446,9 +456,17 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
           if constexpr (TM) {
             if constexpr (HT < H) smem_words(HT / 4);
 #pragma unroll
-            for (int q = HT - 1; q >= 1; q -= 2) {
-              cell(q, Tc[q]);
-              cell(q - 1, Tc[q - 1]);
+            for (int q = HI - 1; q >= 1; q -= 2) {
+              cell(LO + q, thi[q]);
+              cell(LO + q - 1, thi[q - 1]);
+              fold(LO + q - 1);
+            }
+            tm_wait_ld<LOW>(tlo);
+            tm_ld_pow2<HI>(thi, tm_col(rr < 3 ? __byte_perm(cur, 0u, 0x4440u + rr + 1) : nxt & 0xffu) + LO);
+#pragma unroll
+            for (int q = LO - 1; q >= 1; q -= 2) {
+              cell(q, tlo[q]);
+              cell(q - 1, tlo[q - 1]);
               fold(q - 1);
             }
           } else {
@@ -490,18 +508,15 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
               if (exact) vacc = 0u;
             }
           }
-         };
-          if (rr & 1)
-            one_row(TB, TA);
-          else
-            one_row(TA, TB);
+         }
         }
       };
 
       int since_clear = 0;
       for (int step = 0; step < wsteps; ++step) {
-        // Prefetch the next residue word; past the end a group reads padding.
-        const uint32_t nxt = __ldg(p.residues + (step + 1 < nsteps ? wptr + (uint32_t)step + 1u : p.pad_word));
+        // Prefetch the residue words; past the end a group reads padding.
+        const uint32_t nxt = kUniform ? __reduce_max_sync(kFull, ahead) : ahead;
+        ahead = __ldg(p.residues + (step + 2 < nsteps ? wptr + (uint32_t)step + 2u : p.pad_word));
         if (kFast) {
           const bool near = active && !done && (exact || Tnear < 0 || ((vacc + Tnear2) & 0x80008000u) != 0u);
           if (__any_sync(kFull, near))
@@ -523,7 +538,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         }
       }
 
-      if constexpr (TM) tm_wait_ld<HL>(TA);   // the load issued after the last row
+      if constexpr (TM) tm_wait_ld<HI>(thi);   // the load issued after the last row
 
       // ---- finalise the G sequences -------------------------------------
       const bool own = active && qvalid;   // this group writes its sequence's outputs
