@@ -203,6 +203,15 @@ constexpr int kVitRows = 32;         // msc rows: residue codes 0..31
 constexpr int kVitTrans = 8;         // BM, MM, IM, DM, MI, II, MD, DD
 constexpr int kVitSpecial = 8;       // NN, NB, EC, CC, CT, EJ, JJ, JB
 
+// Tables of the packed Viterbi kernel: kVitPackPlanes transition planes (MD,
+// DD, MM, IM, DM, MI, II) of `words` x 32 words, then kVitRows rows of match
+// scores and as many for the second step.
+constexpr int kVitPackPlanes = 7;
+struct VitPackTables {
+  const uint32_t *trans;
+  int words;                  // 64 nodes each
+};
+
 // One query of a Viterbi launch (lives in device memory).
 struct VitQuery {
   const int16_t *msc;         // kVitRows x Mpad match scores (codes >= K: -32768)
@@ -216,6 +225,16 @@ struct VitQuery {
   float *nat;                 // nullable
   const uint32_t *ranks;      // nullable: score only these length ranks (ascending),
   const uint32_t *n_ranks;    //   *n_ranks of them
+  // Packed kernel (mpf_vit_packed.cu), if the query qualifies: tables for one
+  // warp per sequence and for teams (words 0: none); teams score the query
+  // when it selects at most pk_team_max sequences.
+  VitPackTables pk_solo, pk_team;
+  int64_t pk_team_max;
+  int pk_bm, pk_emax, pk_off; // entry move; largest match score, at least 1; first offset
+  uint32_t pk_split;          // residue codes whose match scores are added in two steps
+  int pk_rebase;              // the offset may be lowered
+  uint32_t *fb_ranks;         // sequences left to the 32-bit kernels, and their count
+  uint32_t *fb_count;
   int64_t team_max;           // the team kernel scores the query when it selects at most
                               //   this many sequences, the one-warp kernels otherwise
 };
@@ -232,6 +251,7 @@ struct VitParams {
   int max_Mpad;               // largest Mpad of the queries (sets shared memory)
   const VitQuery *queries;
   uint32_t *counters;         // one per query, zero before the launch
+  int team_warps;             // packed kernel: warps per sequence
   uint2 *state;               // models past the shared-memory rows: per-warp DP rows, else null
   uint64_t state_bytes;
 };
@@ -253,6 +273,24 @@ int64_t viterbi_team_max(int key, int Mpad, int n_codes, int max_smem, int num_s
 // general kernel).  n_seqs: sequences each query of the launch scores, 0
 // when the host does not know (a rank list counted on the device).
 int viterbi_shape_key(bool fast, int Mpad, int n_codes, int max_smem, int num_sms, uint64_t n_seqs);
+
+// Packed Viterbi kernel (mpf_vit_packed.cu): two nodes per register, one warp
+// or a team of `warps` warps per sequence with qh words per lane each.
+constexpr int kVitPackReach = 16384;   // largest decline of one move or match step
+constexpr int kVitPackStep = 8192;     // offset change when the entry score nears the floor
+constexpr int kVitPackShortQH = 8;     // segments up to this many nodes: passing costs in 16 bits
+constexpr int kVitPackRegQH = 8;       // words per lane up to which the transitions stay in registers
+constexpr int kVitPack512QH = 28;      // words per lane up to which blocks have 512 threads
+constexpr int kVitPackMaxSolo = 48;    // words per lane of the longest model one warp takes
+constexpr int kVitPackTeamQH = 5, kVitPackMaxTeamQH = 8;   // words per lane of teams: wanted, at most
+struct VitPackShape {
+  int warps = 0, qh = 0;
+};
+// The shape for a model of M nodes (warps 0: none).
+VitPackShape vit_pack_solo(int M);
+VitPackShape vit_pack_team(int M);
+// Scores the queries of p (all of shape s); returns as launch_viterbi.
+int launch_viterbi_packed(const VitParams &p, VitPackShape s, int max_smem, int num_sms, cudaStream_t st);
 
 // Kernel instantiation for (lanes, words, mode), or nullptr if not built.
 KernelFn kernel_for(int lanes, int words, int mode);
