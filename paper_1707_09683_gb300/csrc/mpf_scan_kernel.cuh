@@ -30,10 +30,11 @@
 // which follows the SSV recurrence while b is constant; b only changes when
 // xJ passes base, so each lane keeps a running maximum and the group reduces
 // it (Alg. 6) only on rows where some lane crosses the threshold at which xJ
-// would pass base or the score would overflow.  After the first such row
-// the group reduces every row (exact mode) until the sequence ends.  A row
-// can raise the running maximum by at most `bias`, so a warp runs four rows
-// without any per-row test whenever no lane is within 4 * bias of T.
+// would pass base or the score would overflow.  Such a row updates xJ and b,
+// rebases the cells and starts over with the threshold at which xJ would
+// change again, so the rows in between stay reduction-free.  Before the first
+// one a row can raise the running maximum by at most `bias`, so a warp runs
+// four rows without any per-row test whenever no lane is within 4 * bias of T.
 //
 // Row pairs (SSV, held MSV and the two together, integer cells).  The kernels
 // are bound by the integer ALU pipe, on which a DPX instruction takes two
@@ -341,14 +342,18 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       int xJ = 0;
       int b = min(sat8(base - (t + tbm)), cap);
       uint32_t b2 = pack2(b << kCellShift);
-      const int T = min(base + tec - b, cap - b - 1);
-      const int Tk = value_key<kF16>(max(T, 0));          // threshold as a key
-      const int Tnear = T - 4 * max(bias, 0);              // no trigger possible in 4 rows below it
-      const int Tnear_k = value_key<kF16>(max(Tnear, 0));
+      int T = min(base + tec - b, cap - b - 1);
+      int Tnear = 0;           // no trigger possible in 4 rows below it
+      uint32_t Tk2 = 0u, Tnear2 = 0u;
       // "Some half of the running maximum is above the key K" as one add and
       // one mask: the halves (keys <= 0x7fff) plus 0x7fff - K reach bit 15
       // exactly when they exceed K, and no sum carries into the other half.
-      const uint32_t Tk2 = pack2(0x7fff - Tk), Tnear2 = pack2(0x7fff - Tnear_k);
+      auto arm = [&]() {
+        Tnear = T - 4 * max(bias, 0);
+        Tk2 = pack2(0x7fff - value_key<kF16>(max(T, 0)));
+        Tnear2 = pack2(0x7fff - value_key<kF16>(max(Tnear, 0)));
+      };
+      if constexpr (kFast) arm();
       bool done = false, exact = false;
 
       // Lane state: H words of two 16-bit cells and a running maximum (key).
@@ -485,15 +490,15 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
               }
             }
           } else if (kFast && CHECK) {
-            const bool trig = real && !done && (exact || ((vacc + Tk2) & 0x80008000u) != 0u);
+            const bool trig = real && !done && ((vacc + Tk2) & 0x80008000u) != 0u;
             if (__any_sync(kFull, trig)) {
               const int mm = key_value<kF16>(group_max<LG>(half_max(vacc)));
-              if (real && !done && (exact || mm > T)) {
+              if (real && !done && mm > T) {
                 const int xE = b + mm;
                 if (xE >= cap) {
                   done = true;
                 } else {
-                  xJ = exact ? max(xJ, xE - tec) : max(0, xE - tec);
+                  xJ = max(xJ, xE - tec);
                   const int bn = min(sat8(max(base, xJ) - (t + tbm)), cap);
                   if (bn > b) {
 #pragma unroll
@@ -503,9 +508,14 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
                   }
                   b = bn;
                   exact = true;
+                  // Lazy again: a later row changes xJ or overflows only with
+                  // a cell above the new threshold (0 or more: b stays below
+                  // cap).  From here on every row is tested.
+                  T = min(xJ + tec - b, cap - b - 1);
+                  arm();
+                  vacc = 0u;
                 }
               }
-              if (exact) vacc = 0u;
             }
           }
          }
