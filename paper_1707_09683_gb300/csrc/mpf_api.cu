@@ -361,7 +361,7 @@ std::vector<std::pair<size_t, size_t>> pack_runs(int lanes, int mode, const std:
 }  // namespace mpf
 
 // One launch of the scan kernel over a set of queries sharing a kernel
-// configuration.  Device arrays are owned by the group.
+// configuration.  Device arrays lie in the plan's allocation.
 struct LaunchGroup {
   KernelFn fn = nullptr;
   int lanes = 0, words = 0, mode = 0;
@@ -378,12 +378,16 @@ struct LaunchGroup {
   uint8_t *d_col = nullptr;      // tiled kernel: two columns of col_stride bytes per resident warp
   uint32_t col_stride = 0;
   uint64_t col_bytes = 0;
-  uint32_t *d_fallback = nullptr;   // tiled MSV: per query a count, then n_seqs ranks per query
+  uint32_t *d_zero = nullptr;       // words zeroed before each launch (null: a fallback launch, zeroed with its group)
+  size_t zero_words = 0;
   bool tm = false;                  // striped kernel with the table in tensor memory
   int shard_factor = 1;             // striped kernels: shards = factor x resident blocks
   uint32_t n_real = 0;              // queries of the group (n_queries less empty slots of packed sets)
   int qp = 1;                       // tensor-memory kernels: queries scored per warp and sequence
   uint32_t qp_stride = 0;           //   and shared-memory bytes per staged table (qp > 1)
+  // Split sequences (plan_split); n_long 0: none.
+  uint32_t n_long = 0, n_long_units = 0, seg_rows = 0, seg_overlap = 0;
+  uint32_t *d_units = nullptr;      // unit_rank, then unit_first
   std::shared_ptr<LaunchGroup> next;   // launched after this group on the same stream
 };
 
@@ -391,6 +395,7 @@ struct mpf_plan {
   mpf_ctx *ctx = nullptr;
   const mpf_db *db = nullptr;
   std::vector<LaunchGroup> groups;
+  uint8_t *d_mem = nullptr;          // everything the groups point to
   std::vector<cudaEvent_t> events;   // fork/join events (more than one group)
   cudaGraphExec_t graph = nullptr;
 };
@@ -402,13 +407,7 @@ void plan_free(mpf_plan *pl) {
   DeviceGuard dg(pl->ctx->device);
   if (pl->graph) cudaGraphExecDestroy(pl->graph);
   // Ordered after the plan's last launch, which joins back into this stream.
-  for (auto &g0 : pl->groups)
-    for (LaunchGroup *g = &g0; g; g = g->next.get()) {
-      if (g->d_queries) cudaFreeAsync(g->d_queries, pl->ctx->stream);
-      if (g->d_counter) cudaFreeAsync(g->d_counter, pl->ctx->stream);
-      if (g->d_col) cudaFreeAsync(g->d_col, pl->ctx->stream);
-      if (g->d_fallback) cudaFreeAsync(g->d_fallback, pl->ctx->stream);
-    }
+  if (pl->d_mem) cudaFreeAsync(pl->d_mem, pl->ctx->stream);
   for (auto e : pl->events) cudaEventDestroy(e);
   (void)cudaGetLastError();
   delete pl;
@@ -519,6 +518,66 @@ int configure_kernel(mpf_ctx *ctx, LaunchGroup *g) {
   g->grid = ctx->num_sms * per_sm;
   g->n_shards = (uint32_t)g->grid * (uint32_t)std::max(1, g->shard_factor);
   return MPF_OK;
+}
+
+// Work of a launch group per residue, in words of a warp.
+double group_work(const LaunchGroup &g, const std::vector<QueryDesc> &queries) {
+  if (g.words)
+    return (double)((queries.size() + g.qp - 1) / g.qp) * g.words * (g.qp > 1 ? 1.0 : g.lanes / 32.0);
+  double w = 0;
+  for (const QueryDesc &q : queries) w += q.M / 64.0;
+  return w;
+}
+
+// Decide which sequences a launch group over the whole database scores in
+// segments; returns its unit tables (empty: none is split).  With the longest
+// units first, a plan lasts about its rows per lane group (n_rows below: all
+// sequences spread evenly, and the time of its other launch groups in rows of
+// this one) or its longest unit.  So sequences longer than n_rows are cut to
+// that, but to no fewer rows than the longest model has nodes (each segment
+// also reads that many rows before it) or kMinSegRows; a little longer than
+// that they stay whole.  Segments get longer until the rows read twice are at
+// most a kMaxAddedRows-th of the database (they cost time when other streams
+// keep the device busy: with segments of 128 rows and M = 100, 10,000
+// sequences took 254 us per pass among others, against 195 whole).  share:
+// the part of the plan's work (group_work) that is this group's.  Measured (MSV + SSV of one query, alone on the device):
+// 6,001 sequences with twelve of 5,000-35,000 residues, M = 777: 3.83 -> 0.62
+// ms; 1,000 sequences of up to 2,000, M = 100: 414 -> 275 us.
+constexpr uint32_t kMinSegRows = 128;
+constexpr uint64_t kMaxAddedRows = 12;
+std::vector<uint32_t> plan_split(const mpf_db *db, double share, const std::vector<QueryDesc> &queries,
+                                 LaunchGroup *g) {
+  if (db->longest.empty()) return {};
+  uint32_t M = 1;
+  for (const QueryDesc &q : queries) M = std::max(M, q.M);
+  const uint64_t per_warp = g->qp > 1 ? 1 : 32 / (uint64_t)g->lanes;
+  const uint64_t groups = (uint64_t)g->grid * (kBlockThreads / 32) * per_warp;
+  const uint64_t sets = ((uint64_t)queries.size() + g->qp - 1) / g->qp;
+  const uint64_t n_rows = (uint64_t)((double)(sets * db->n_residues / groups) / share);
+  uint64_t S = std::max<uint64_t>({n_rows, M, kMinSegRows});
+  const auto &len = db->longest;
+  for (;; S += S / 2) {
+    S = (S + 3) & ~(uint64_t)3;
+    if (S + S / 4 >= len[0]) return {};
+    if (len.back() > S && len.size() < db->n_seqs) return {};   // lengths not kept: no short launch
+    uint64_t added = 0;
+    for (size_t r = 0; r < len.size() && len[r] > S && kMaxAddedRows * added <= db->n_residues; ++r)
+      added += (len[r] - 1) / S * M;
+    if (kMaxAddedRows * added <= db->n_residues) break;
+  }
+  std::vector<uint32_t> host;   // unit_rank, then (below) unit_first
+  std::vector<uint32_t> first{0};
+  for (uint32_t r = 0; r < len.size() && len[r] > S; ++r) {
+    const uint32_t n = (uint32_t)((len[r] + S - 1) / S);
+    host.insert(host.end(), n, r);
+    first.push_back((uint32_t)host.size());
+  }
+  g->n_long = (uint32_t)first.size() - 1;
+  g->n_long_units = (uint32_t)host.size();
+  g->seg_rows = (uint32_t)S;
+  g->seg_overlap = (M + 3) & ~3u;
+  host.insert(host.end(), first.begin(), first.end());
+  return host;
 }
 
 // Build a plan: queries grouped by kernel configuration.
@@ -734,6 +793,29 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     }
   }
   DeviceGuard dg(ctx->device);
+  // Byte offsets of a group's parts in the plan's device memory: of the
+  // uploaded part, and of the rest.
+  struct Parts {
+    size_t desc = 0, fb_desc = 0, unit_tables = 0, zero = 0, fb_ranks = 0, unit_max = 0, col = 0;
+    std::vector<uint32_t> units;
+  };
+  struct Layout {
+    size_t bytes = 0;
+    size_t take(size_t n) {
+      const size_t at = bytes;
+      bytes += (n + 255) & ~(size_t)255;
+      return at;
+    }
+  } up, rest;
+  std::vector<Parts> parts;
+  double work = 0;
+  for (auto &kv : byconf) {
+    LaunchGroup g;
+    g.lanes = std::get<0>(kv.first);
+    g.words = std::get<1>(kv.first);
+    g.qp = std::get<4>(kv.first);
+    work += group_work(g, kv.second);
+  }
   for (auto &kv : byconf) {
     LaunchGroup g;
     g.lanes = std::get<0>(kv.first);
@@ -753,76 +835,117 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     }
     g.n_queries = (uint32_t)kv.second.size();
     for (const QueryDesc &qd : kv.second) g.n_real += qd.table ? 1u : 0u;
-    cudaError_t e = cudaMallocAsync((void **)&g.d_queries, sizeof(QueryDesc) * kv.second.size(), ctx->stream);
-    if (e == cudaSuccess) e = cudaMallocAsync((void **)&g.d_counter, sizeof(uint32_t), ctx->stream);
-    if (e == cudaSuccess && (g.mode == MODE_TILE_SSV || g.mode == MODE_TILE_MSV || g.mode == MODE_TILE_MSV_SSV)) {
+    const size_t nq = kv.second.size(), ns = std::max<uint64_t>(db->n_seqs, 1);
+    const bool tiled = g.mode == MODE_TILE_SSV || g.mode == MODE_TILE_MSV || g.mode == MODE_TILE_MSV_SSV;
+    const bool held = g.mode == MODE_MSV_HELD || g.mode == MODE_MSV_HELD_F16 || g.mode == MODE_MSV_SSV;
+    const bool fallback = held || g.mode == MODE_TILE_MSV || g.mode == MODE_TILE_MSV_SSV;
+    Parts pt;
+    if (!ranks && (held || g.mode == MODE_SSV || g.mode == MODE_SSV_F16))
+      pt.units = plan_split(db, group_work(g, kv.second) / work, kv.second, &g);
+    if (tiled) {
       // Per resident warp two columns (positions 0..max_len and the
       // prefetch's overrun), col_stride bytes each: int16, or for the TMEM
       // kernel the 32-bit pair holding the node.
       g.col_stride = (uint32_t)((((uint64_t)db->max_len + 12) * (g.tm ? 4 : 2) + 15) & ~(uint64_t)15);
       g.col_bytes = (uint64_t)g.grid * (uint64_t)(g.threads / 32) * 2 * g.col_stride;
-      e = cudaMallocAsync((void **)&g.d_col, g.col_bytes, ctx->stream);
     }
-    const bool held = g.mode == MODE_MSV_HELD || g.mode == MODE_MSV_HELD_F16 || g.mode == MODE_MSV_SSV;
-    if (e == cudaSuccess && (g.mode == MODE_TILE_MSV || g.mode == MODE_TILE_MSV_SSV || held)) {
+    if (fallback) {
       // Fallback lists, and the launch that scores them exactly: the
       // lane-segment kernel after the tiled MSV pass, the striped kernel
-      // with the J/B update every row after the held pass.
+      // that follows xJ and xB after the held pass.
+      auto nx = std::make_shared<LaunchGroup>();
+      // MSV_FAST reduces only the rows that change xJ; MSV_DIRECT, which
+      // reduces every row, took 1.2 to 1.8 times as long on these few
+      // sequences (M = 100-2405, 80,000 sequences: 156-352 us against
+      // 132-260).
+      nx->mode = held ? MODE_MSV_FAST : MODE_LONG_MSV;
+      nx->lanes = g.lanes;
+      nx->words = g.words;
+      nx->n_codes = db->n_codes;
+      nx->n_long = g.n_long;
+      nx->n_long_units = g.n_long_units;
+      nx->seg_rows = g.seg_rows;
+      nx->seg_overlap = g.seg_overlap;
+      for (size_t i = 0; i < nq; ++i) {   // the group's queries (not the empty slots of packed sets)
+        if (!kv.second[i].table) continue;
+        ++nx->n_queries;
+        if (!held) nx->long_words = std::max(nx->long_words, fb_seg_words[kv.first][i]);
+      }
+      nx->n_real = nx->n_queries;
+      int rc2 = configure_kernel(ctx, nx.get());
+      if (rc2) {
+        plan_free(pl);
+        return rc2;
+      }
+      g.next = nx;
+    }
+    // What is uploaded (descriptors, unit tables), what is zeroed before each
+    // launch (the work counters of the group and its fallback launch, the
+    // fallback counts, the finished units), and scratch.
+    pt.desc = up.take(sizeof(QueryDesc) * nq);
+    pt.fb_desc = up.take(fallback ? sizeof(QueryDesc) * g.next->n_queries : 0);
+    pt.unit_tables = up.take(4 * pt.units.size());
+    g.zero_words = 2 + (fallback ? nq : 0) + nq * g.n_long;
+    pt.zero = rest.take(4 * g.zero_words);
+    pt.fb_ranks = rest.take(fallback ? 4 * nq * ns : 0);
+    pt.unit_max = rest.take(4 * nq * g.n_long_units);
+    pt.col = rest.take(g.col_bytes);
+    parts.push_back(std::move(pt));
+    pl->groups.push_back(g);
+  }
+  // One stream-ordered allocation and one copy for the whole plan.
+  cudaError_t e = cudaMallocAsync((void **)&pl->d_mem, up.bytes + rest.bytes, ctx->stream);
+  if (e == cudaSuccess) {
+    std::vector<uint8_t> host(up.bytes);
+    uint8_t *base = pl->d_mem, *scratch = pl->d_mem + up.bytes;
+    size_t gi = 0;
+    for (auto &kv : byconf) {
+      LaunchGroup &g = pl->groups[gi];
+      const Parts &pt = parts[gi++];
       const size_t nq = kv.second.size(), ns = std::max<uint64_t>(db->n_seqs, 1);
-      e = cudaMallocAsync((void **)&g.d_fallback, (nq + nq * ns) * 4, ctx->stream);
-      if (e == cudaSuccess) {
-        auto nx = std::make_shared<LaunchGroup>();
-        // MSV_FAST reduces only the rows that change xJ; MSV_DIRECT, which
-        // reduces every row, took 1.2 to 1.8 times as long on these few
-        // sequences (M = 100-2405, 80,000 sequences: 156-352 us against
-        // 132-260).
-        nx->mode = held ? MODE_MSV_FAST : MODE_LONG_MSV;
-        nx->lanes = g.lanes;
-        nx->words = g.words;
-        nx->n_codes = db->n_codes;
-        std::vector<QueryDesc> fq;   // the group's queries (not the empty slots of packed sets)
-        for (size_t i = 0; i < nq; ++i) {
-          kv.second[i].fallback_count = g.d_fallback + i;
-          kv.second[i].fallback_ranks = g.d_fallback + nq + i * ns;
-          if (!kv.second[i].table) continue;
-          QueryDesc f = kv.second[i];
-          if (held) {
-            set_table(f, fb_table[kv.first][i]);
-          } else {
-            f.table = fb_table[kv.first][i].ptr;
-            f.seg_words = fb_seg_words[kv.first][i];
-          }
-          f.ranks = kv.second[i].fallback_ranks;
-          f.n_ranks = kv.second[i].fallback_count;
-          nx->long_words = std::max(nx->long_words, f.seg_words);
-          fq.push_back(f);
+      uint32_t *zero = reinterpret_cast<uint32_t *>(scratch + pt.zero);
+      uint32_t *fb_count = zero + 2, *unit_done = fb_count + (g.next ? nq : 0);
+      uint32_t *fb_ranks = reinterpret_cast<uint32_t *>(scratch + pt.fb_ranks);
+      int *unit_max = reinterpret_cast<int *>(scratch + pt.unit_max);
+      g.d_queries = reinterpret_cast<QueryDesc *>(base + pt.desc);
+      g.d_counter = g.d_zero = zero;
+      g.d_col = g.col_bytes ? scratch + pt.col : nullptr;
+      g.d_units = reinterpret_cast<uint32_t *>(base + pt.unit_tables);
+      if (!pt.units.empty()) memcpy(&host[pt.unit_tables], pt.units.data(), 4 * pt.units.size());
+      std::vector<QueryDesc> fq;
+      for (size_t i = 0; i < nq; ++i) {
+        QueryDesc &q = kv.second[i];
+        q.unit_done = unit_done + i * g.n_long;
+        q.unit_max = unit_max + i * g.n_long_units;
+        if (!g.next) continue;
+        q.fallback_count = fb_count + i;
+        q.fallback_ranks = fb_ranks + i * ns;
+        if (!q.table) continue;
+        QueryDesc f = q;
+        if (g.next->mode == MODE_LONG_MSV) {
+          f.table = fb_table[kv.first][i].ptr;
+          f.seg_words = fb_seg_words[kv.first][i];
+        } else {
+          set_table(f, fb_table[kv.first][i]);
         }
-        g.next = nx;
-        int rc2 = configure_kernel(ctx, nx.get());
-        if (rc2) {
-          pl->groups.push_back(g);
-          plan_free(pl);
-          return rc2;
-        }
-        nx->n_queries = (uint32_t)fq.size();
-        nx->n_real = nx->n_queries;
-        e = cudaMallocAsync((void **)&nx->d_queries, sizeof(QueryDesc) * fq.size(), ctx->stream);
-        if (e == cudaSuccess) e = cudaMallocAsync((void **)&nx->d_counter, sizeof(uint32_t), ctx->stream);
-        if (e == cudaSuccess)
-          e = cudaMemcpyAsync(nx->d_queries, fq.data(), sizeof(QueryDesc) * fq.size(),
-                              cudaMemcpyHostToDevice, ctx->stream);
+        f.ranks = q.fallback_ranks;
+        f.n_ranks = q.fallback_count;
+        fq.push_back(f);
+      }
+      memcpy(&host[pt.desc], kv.second.data(), sizeof(QueryDesc) * nq);
+      if (g.next) {
+        memcpy(&host[pt.fb_desc], fq.data(), sizeof(QueryDesc) * fq.size());
+        g.next->d_queries = reinterpret_cast<QueryDesc *>(base + pt.fb_desc);
+        g.next->d_counter = zero + 1;
+        g.next->d_units = g.d_units;
       }
     }
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(g.d_queries, kv.second.data(), sizeof(QueryDesc) * kv.second.size(),
-                          cudaMemcpyHostToDevice, ctx->stream);
-    if (e != cudaSuccess) {
-      (void)cudaGetLastError();
-      pl->groups.push_back(g);   // plan_free releases what the group holds
-      plan_free(pl);
-      return e == cudaErrorMemoryAllocation ? MPF_ENOMEM : MPF_ECUDA;
-    }
-    pl->groups.push_back(g);
+    e = cudaMemcpyAsync(pl->d_mem, host.data(), up.bytes, cudaMemcpyHostToDevice, ctx->stream);
+  }
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    plan_free(pl);
+    return e == cudaErrorMemoryAllocation ? MPF_ENOMEM : MPF_ECUDA;
   }
   if (pl->groups.size() > 1) {
     while (ctx->n_fork < 8 && (size_t)ctx->n_fork < pl->groups.size()) {
@@ -848,8 +971,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
 }
 
 int enqueue_group(const mpf_db *db, mpf_ctx *ctx, LaunchGroup &g, cudaStream_t st) {
-  MPF_CUDA(cudaMemsetAsync(g.d_counter, 0, sizeof(uint32_t), st));
-  if (g.d_fallback) MPF_CUDA(cudaMemsetAsync(g.d_fallback, 0, sizeof(uint32_t) * g.n_queries, st));
+  if (g.d_zero) MPF_CUDA(cudaMemsetAsync(g.d_zero, 0, 4 * g.zero_words, st));
   ScanParams sp{};
   sp.residues = db->d_words;
   sp.n_words = db->n_words;
@@ -870,6 +992,13 @@ int enqueue_group(const mpf_db *db, mpf_ctx *ctx, LaunchGroup &g, cudaStream_t s
   sp.qp_table_stride = g.qp_stride;
   sp.one = 1;
   sp.tm_rows = g.tm_rows;
+  sp.n_long = g.n_long;
+  sp.n_long_units = g.n_long_units;
+  sp.n_units = sp.n_seqs - g.n_long + g.n_long_units;
+  sp.seg_rows = g.seg_rows;
+  sp.seg_overlap = g.seg_overlap;
+  sp.unit_rank = g.d_units;
+  sp.unit_first = g.d_units + g.n_long_units;
   const uint64_t n_items = ((uint64_t)g.n_queries + (uint64_t)g.qp - 1) / (uint64_t)g.qp * g.n_shards;
   const int grid = (int)std::min<uint64_t>((uint64_t)g.grid, n_items);
   g.fn<<<grid, g.threads, g.smem, st>>>(sp);
@@ -1269,6 +1398,8 @@ int mpf_db_upload(mpf_ctx *ctx, const uint8_t *residues, uint64_t n_residues,
   db->n_codes = __builtin_popcount(seen);
   db->code_end = seen ? 32 - __builtin_clz(seen) : 1;
   db->max_len = n_seqs ? seq_len[0] : 0;
+  constexpr uint64_t kHostLengths = 1u << 20;
+  db->longest.assign(seq_len.begin(), seq_len.begin() + (ptrdiff_t)std::min<uint64_t>(n_seqs, kHostLengths));
   const size_t ns = std::max<uint64_t>(n_seqs, 1);
   db->n_words = (uint32_t)(chunks * 4);
   cudaError_t e = cudaMalloc(&db->d_words, chunks * 16);

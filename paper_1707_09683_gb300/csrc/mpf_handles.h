@@ -72,6 +72,7 @@ struct mpf_db {
   uint32_t pad_word = 0;
   int n_codes = 0;                  // distinct residue codes present
   int code_end = 32;                // largest residue code present + 1
+  std::vector<uint32_t> longest;    // lengths of the first length ranks (up to kHostLengths)
   uint32_t max_len = 0;             // longest sequence
 };
 

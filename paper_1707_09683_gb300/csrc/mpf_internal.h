@@ -123,6 +123,10 @@ struct QueryDesc {
   // length ranks, and the count, zero before the launch).
   uint32_t *fallback_ranks;
   uint32_t *fallback_count;
+  // Split sequences (striped kernels): each unit's largest cell, and per rank
+  // the units that have finished (zero before the launch).
+  int *unit_max;
+  uint32_t *unit_done;
 };
 
 struct ScanParams {
@@ -142,6 +146,12 @@ struct ScanParams {
   uint8_t *tile_col;          // tiled kernel: per resident warp two columns of
   uint32_t tile_col_stride;   //   tile_col_stride bytes (an int16 per row)
   uint64_t tile_col_bytes;
+  // Work units of the striped kernels without rank lists: first the segments
+  // of ranks 0 .. n_long - 1 (unit u belongs to rank unit_rank[u], whose
+  // units start at unit_first[rank]; seg_rows rows each, read from
+  // seg_overlap rows before), then the other ranks whole.
+  uint32_t n_units, n_long, n_long_units, seg_rows, seg_overlap;
+  const uint32_t *unit_rank, *unit_first;
   uint32_t tm_rows;           // TM_FEW kernels: TMEM rows, the database's codes and the padding code
   uint32_t one;               // 1 (striped kernels: see add_imad)
   uint32_t qp_table_stride;   // striped kernels with several queries per warp: bytes per staged table

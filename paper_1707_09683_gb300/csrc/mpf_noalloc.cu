@@ -122,6 +122,7 @@ extern "C" int mpf_scan_noalloc(mpf_ctx *ctx, int filter, const mpf_profile *pro
 
   ScanParams sp{};
   sp.one = 1;
+  sp.n_units = (uint32_t)db->n_seqs;
   sp.residues = db->d_words;
   sp.n_words = db->n_words;
   sp.seq_word = db->d_seq_word;

@@ -53,6 +53,22 @@
 // (GB300, clock64, 16 words per lane, table in registers): 52.7 words per
 // clock and SM against 42.4 for two rows of add-then-max.
 //
+// Segments.  A path of the SSV recurrence (and of held MSV, the same cells)
+// visits at most M rows, so the largest cell of rows a .. b - 1 is known from
+// a zero row M rows before a: a long sequence splits into segments of
+// seg_rows rows that different groups score, each with seg_overlap >= M rows
+// before it.  The units' maxima are combined by the last unit to finish
+// (a counter per sequence), which writes the outputs.  Without this a launch
+// ends with its longest sequences, one lane group each: 35,000 residues took
+// milliseconds on a database that needs a tenth of one otherwise.  The host
+// splits only sequences longer than the launch's rows per lane group
+// (plan_split in mpf_api.cu), where the rows added by the overlap run on
+// lanes that would idle.  MSV_FAST rescores such a sequence segment by
+// segment, in order, and skips the segments whose largest cell is at most T:
+// with b constant over a segment no row of it can change xJ.  A segment
+// entered after a gap starts from a zero row seg_overlap <= seg_rows rows
+// earlier, in the skipped segment, over which b did not change either.
+//
 // The F16 modes hold the same integers as IEEE half values and update a cell
 // pair with one fused add-and-clamp-at-zero (HFMA2.RELU, v * 1 + s), which
 // issues on the FMA pipe instead of the integer ALU pipe that the DPX
@@ -182,6 +198,8 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   constexpr bool kBoth = (MODE == MODE_MSV_SSV);   // held MSV and SSV outputs from one sweep
   constexpr bool kHeld = (MODE == MODE_MSV_HELD || MODE == MODE_MSV_HELD_F16 || kBoth);
   constexpr bool kDirect = (MODE == MODE_MSV_DIRECT);
+  // Modes that may take a sequence in segments (see the file comment).
+  constexpr bool kUnits = kSSV || kHeld;
   // SSV and held MSV with integer cells: rows in pairs (see the file comment).
   constexpr bool kPair = !kF16 && (kSSV || kHeld);
   const uint32_t one2 = 0x3c003c00u;   // (1.0, 1.0) as half2
@@ -244,7 +262,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
     }
     // A shard without sequences (a short rank list, such as the few
     // sequences a held MSV pass leaves for rescoring) stages nothing.
-    if ((uint64_t)shard >= (qd->ranks ? (uint64_t)*qd->n_ranks : (uint64_t)p.n_seqs)) {
+    if ((uint64_t)shard >= (qd->ranks ? (uint64_t)*qd->n_ranks : (uint64_t)p.n_units)) {
       __syncthreads();
       continue;
     }
@@ -307,7 +325,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
     const uint32_t tail_row_bytes = qd->tail_row_bytes;
     const int16_t *smax = reinterpret_cast<const int16_t *>(tbl_base + qd->smax_off);
     const uint32_t *ranks = qd->ranks;
-    const uint64_t n_sel = ranks ? (uint64_t)*qd->n_ranks : (uint64_t)p.n_seqs;
+    const uint64_t n_sel = ranks ? (uint64_t)*qd->n_ranks : (uint64_t)p.n_units;
 
     for (;;) {
       // ---- take G consecutive length ranks of this shard (one per group;
@@ -318,7 +336,10 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       const uint64_t kr = (uint64_t)shard + (uint64_t)(k0 + (QP > 1 ? 0 : grp)) * p.n_shards;
       bool active = kr < n_sel;
       if (!__any_sync(kFull, active)) break;
-      const uint64_t r = (ranks && active) ? (uint64_t)__ldg(ranks + kr) : kr;
+      // The first units are the segments of the longest sequences.
+      uint64_t r = (ranks && active) ? (uint64_t)__ldg(ranks + kr) : kr - p.n_long_units + p.n_long;
+      const bool split = kUnits && !ranks && active && kr < p.n_long_units;
+      if (split) r = (uint64_t)__ldg(p.unit_rank + kr);
       if (active && !MPF_DCHECK(p.status, r < p.n_seqs)) active = false;
 
       // Group state (identical in every lane of a group).
@@ -337,8 +358,14 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         }
       }
       const uint32_t wstart = wptr;
-      const int nsteps = (len + 3) >> 2;           // residue words of this sequence
-      const int wsteps = (int)__reduce_max_sync(kFull, (uint32_t)nsteps);
+      // Rows first_row .. first_row + rows - 1: the whole sequence, or this
+      // unit's segment after the rows that its paths can come from.
+      int first_row = 0, rows = len;
+      if (split) {
+        const int end = ((int)(kr - __ldg(p.unit_first + r)) + 1) * (int)p.seg_rows;
+        first_row = max(end - (int)(p.seg_rows + p.seg_overlap), 0);
+        rows = min(end, len) - first_row;
+      }
       int xJ = 0;
       int b = min(sat8(base - (t + tbm)), cap);
       uint32_t b2 = pack2(b << kCellShift);
@@ -361,10 +388,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
 #pragma unroll
       for (int q = 0; q < H; ++q) v[q] = 0u;
       uint32_t vacc = 0u;
-      uint32_t cur = __ldg(p.residues + (nsteps > 0 ? wptr : p.pad_word));
-      if constexpr (kUniform) cur = __reduce_max_sync(kFull, cur);
-      // The residue word after cur, as loaded.
-      uint32_t ahead = __ldg(p.residues + (1 < nsteps ? wptr + 1u : p.pad_word));
+      int nsteps = 0;          // residue words of the rows
+      bool busy = active;      // this group has rows to score
+      uint32_t cur = 0u, ahead = 0u;   // the current residue word, and the next one as loaded
 
       // Tensor-memory words of a row come in two loads, the low words and the
       // high words (processed first, after the words in shared memory); each
@@ -380,8 +406,6 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         if (!MPF_DCHECK(p.status, xc < (uint32_t)kTableRows)) xc = kPadCode;
         return tm_lane + (TM == TM_FEW ? min(xc, tm_pad) : xc) * (uint32_t)HT;
       };
-      if constexpr (TM) tm_ld_pow2<HI>(thi, tm_col(cur & 0xffu) + LO);   // first row of the sequence
-
       // Four rows of one residue word (nxt: the next word).  CHECK: test every
       // row for the MSV threshold (only needed when some lane is near it, or
       // in exact mode).
@@ -392,7 +416,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
          {
           // Rows past the end of a sequence read padding codes: their cells
           // score kNegInf, and the special states must not see them.
-          const bool real = active && (4 * step + rr) < len;
+          const bool real = busy && (4 * step + rr) < rows;
           uint32_t x = __byte_perm(cur, 0u, 0x4440u + rr);   // residue code of row rr
           if (!MPF_DCHECK(p.status, x < (uint32_t)kTableRows)) x = kPadCode;
           if constexpr (TM) {
@@ -522,13 +546,51 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         }
       };
 
+      // A rescored sequence that was split takes its segments one by one and
+      // leaves out those whose largest cell cannot move xJ (see kUnits).
+      int seg = 0;
+      bool follows = false;
+      const int n_segs = kFast && active && r < p.n_long ? (int)(__ldg(p.unit_first + r + 1) - __ldg(p.unit_first + r)) : 1;
+      for (;;) {
+      if constexpr (kFast) {
+        busy = false;
+        if (active && !done) {
+          while (n_segs > 1 && seg < n_segs && __ldcg(qd->unit_max + __ldg(p.unit_first + r) + seg) <= T) {
+            ++seg;
+            follows = false;
+          }
+          if (seg < n_segs) {
+            busy = true;
+            if (n_segs > 1) {
+              const int end = (seg + 1) * (int)p.seg_rows;
+              first_row = max(end - (int)(p.seg_rows + (follows ? 0u : p.seg_overlap)), 0);
+              rows = min(end, len) - first_row;
+            }
+            if (!follows) {
+#pragma unroll
+              for (int q = 0; q < H; ++q) v[q] = 0u;
+            }
+            ++seg;
+            follows = true;
+          }
+        }
+        if (!__any_sync(kFull, busy)) break;
+      }
+      nsteps = busy ? (rows + 3) >> 2 : 0;
+      wptr = busy ? wstart + ((uint32_t)first_row >> 2) : p.pad_word;
+      const int wsteps = (int)__reduce_max_sync(kFull, (uint32_t)nsteps);
+      cur = __ldg(p.residues + (nsteps > 0 ? wptr : p.pad_word));
+      if constexpr (kUniform) cur = __reduce_max_sync(kFull, cur);
+      ahead = __ldg(p.residues + (1 < nsteps ? wptr + 1u : p.pad_word));
+      if constexpr (TM) tm_ld_pow2<HI>(thi, tm_col(cur & 0xffu) + LO);   // first row
+
       int since_clear = 0;
       for (int step = 0; step < wsteps; ++step) {
         // Prefetch the residue words; past the end a group reads padding.
         const uint32_t nxt = kUniform ? __reduce_max_sync(kFull, ahead) : ahead;
         ahead = __ldg(p.residues + (step + 2 < nsteps ? wptr + (uint32_t)step + 2u : p.pad_word));
         if (kFast) {
-          const bool near = active && !done && (exact || Tnear < 0 || ((vacc + Tnear2) & 0x80008000u) != 0u);
+          const bool near = busy && !done && (exact || Tnear < 0 || ((vacc + Tnear2) & 0x80008000u) != 0u);
           if (__any_sync(kFull, near))
             four_rows(step, std::true_type{}, nxt);
           else
@@ -549,17 +611,39 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       }
 
       if constexpr (TM) tm_wait_ld<HI>(thi);   // the load issued after the last row
+      if constexpr (!kFast) break;
+      }
 
       // ---- finalise the G sequences -------------------------------------
-      const bool own = active && qvalid;   // this group writes its sequence's outputs
-      const int V = key_value<kF16>(group_max<LG>(half_max(vacc)));
+      bool own = active && qvalid;   // this group writes its sequence's outputs
+      int V = key_value<kF16>(group_max<LG>(half_max(vacc)));
+      if (kUnits && __any_sync(kFull, split)) {
+        // Of a split sequence's units the last one to finish goes on, with
+        // the largest cell of all of them.
+        uint32_t first = 0, n = 0, last = 1;
+        if (split && own) {
+          first = __ldg(p.unit_first + r);
+          n = __ldg(p.unit_first + r + 1) - first;
+          if (gl == 0) {
+            __stcg(qd->unit_max + kr, V);
+            __threadfence();
+            last = atomicAdd(qd->unit_done + r, 1u) == n - 1u ? 1u : 0u;
+            __threadfence();
+          }
+        }
+        last = __shfl_sync(kFull, last, lane - gl);
+        own = own && last;
+        if (split && own)
+          for (uint32_t u = gl; u < n; u += LG) V = max(V, __ldcg(qd->unit_max + first + u));
+        V = group_max<LG>(V);
+      }
       if (kFast || kHeld) {
         // A sequence whose cells never rose above the begin score: its best
         // row maximum is the best single-cell score of its residues.
-        const bool rescue = active && !done && !exact && V == 0 && len > 0;
+        const bool rescue = own && !done && !exact && V == 0 && len > 0;
         int g = INT_MIN / 2;
         if (rescue) {
-          for (int w = gl; w < nsteps; w += LG) {
+          for (int w = gl; w < (len + 3) >> 2; w += LG) {
             const uint32_t word = __ldg(p.residues + wstart + (uint32_t)w);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
