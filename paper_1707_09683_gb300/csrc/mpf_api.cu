@@ -227,10 +227,11 @@ int get_long_table(const mpf_profile *p, const uint8_t **out) {
 // kTileNodes nodes, [code][chunk][lane] x 4 pairs of int16, lane l's pair
 // p = (node l * kTileC + p, the same + kTileC / 2) of the tile, chunk p / 4;
 // s = bias - cost (codes >= K cost 255), -32768 past M; then the 32 per-code
-// maxima of s over the model.
-int get_tile_table(const mpf_profile *p, const uint4 **out) {
+// maxima of s over the model.  scaled (the tensor-memory kernel): scores in
+// units of 2^kCellShift, kNegInf past M.
+int get_tile_table(const mpf_profile *p, bool scaled, const uint4 **out) {
   std::lock_guard<std::mutex> lk(p->mu);
-  auto key = std::make_tuple(32, 0, 3);
+  auto key = std::make_tuple(32, 0, scaled ? 4 : 3);
   auto it = p->tables.find(key);
   if (it != p->tables.end()) {
     *out = it->second.ptr;
@@ -250,8 +251,11 @@ int get_tile_table(const mpf_profile *p, const uint4 **out) {
       for (int l = 0; l < 32; ++l)
         for (int c = 0; c < kTileC; ++c) {
           const int k = t * kTileNodes + l * kTileC + c;
-          int16_t s = -32768;
-          if (k < M) s = (int16_t)(p->bias - (x < p->K ? (int)p->cost[(size_t)x * M + k] : 255));
+          int16_t s = (int16_t)(scaled ? kNegInf : -32768);
+          if (k < M) {
+            const int sv = p->bias - (x < p->K ? (int)p->cost[(size_t)x * M + k] : 255);
+            s = (int16_t)(scaled ? sv * (1 << kCellShift) : sv);
+          }
           const int pr = c % (kTileC / 2), half = c / (kTileC / 2);
           const size_t chunk = (((size_t)t * 32 + x) * kChunks + pr / 4) * 32 + l;
           img[chunk * 8 + (pr % 4) * 2 + half] = s;
@@ -650,7 +654,8 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     int lanes = 32, words = 0;
     if (mode == MODE_TILE_SSV || mode == MODE_TILE_MSV || mode == MODE_TILE_MSV_SSV) {
       const uint4 *tt = nullptr;
-      int rc = get_tile_table(p, &tt);
+      const int ttm = p->table_mem[f] == MPF_TABLE_SHARED ? 0 : 1;   // tiles in TMEM
+      int rc = get_tile_table(p, ttm != 0, &tt);
       if (rc) {
         plan_free(pl);
         return rc;
@@ -658,7 +663,6 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       q.table = tt;
       q.M = (uint32_t)p->M;
       q.smax_off = (uint32_t)(((size_t)(p->M + kTileNodes - 1) / kTileNodes) * kTileTableBytes);
-      const int ttm = p->table_mem[f] == MPF_TABLE_SHARED ? 0 : 1;   // tiles in TMEM
       if (mode != MODE_TILE_SSV) {   // the lane-segment kernel's table, for the fallback
         const uint8_t *lt = nullptr;
         rc = get_long_table(p, &lt);

@@ -14,6 +14,15 @@ constexpr int kStatusBadIndex = 2;
 __device__ __forceinline__ void report_bad_index(int *status) {
   if (status) atomicCAS(status, 0, kStatusBadIndex);
 }
+// a + b as one 32-bit multiply-add (a * one + b, one = 1 in a register the
+// compiler does not see through): it issues on the FMA pipe, beside the
+// integer ALU pipe of the DPX instructions.
+__device__ __forceinline__ uint32_t add_imad(uint32_t a, uint32_t b, uint32_t one) {
+  uint32_t r;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(one), "r"(b));
+  return r;
+}
+
 // Dynamic shared memory of the running block, in bytes.
 __device__ __forceinline__ uint32_t dynamic_smem_bytes() {
   uint32_t r;

@@ -163,15 +163,6 @@ __device__ __forceinline__ uint32_t hfma2_relu_u32(uint32_t a, uint32_t b, uint3
   return *reinterpret_cast<const uint32_t *>(&r);
 }
 
-// a + b as one 32-bit multiply-add (a * one + b, one = 1 in a register the
-// compiler does not see through): it issues on the FMA pipe, beside the
-// integer ALU pipe of the DPX instructions.
-__device__ __forceinline__ uint32_t add_imad(uint32_t a, uint32_t b, uint32_t one) {
-  uint32_t r;
-  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(one), "r"(b));
-  return r;
-}
-
 __device__ __forceinline__ uint32_t pack2_half(int v) {
   const uint32_t h = (uint32_t)__half_as_ushort(__int2half_rn(v));
   return (h << 16) | h;

@@ -84,48 +84,39 @@ __device__ __forceinline__ void tile_row(uint32_t (&v)[kPairs], uint32_t in, con
   }
 }
 
-// tile_row with the row's scores in registers (word p = pair p).
-__device__ __forceinline__ void tile_row_regs(uint32_t (&v)[kPairs], uint32_t in, const uint32_t (&sc)[kPairs],
-                                              uint32_t &rmax) {
-  const uint32_t d0 = __byte_perm(in, v[kPairs - 1], 0x5410);
-#pragma unroll
-  for (int q = kChunks - 1; q >= 0; --q) {
-#pragma unroll
-    for (int e = 3; e >= 0; --e) {
-      const int p = q * 4 + e;
-      v[p] = __viaddmax_s16x2(p > 0 ? v[p - 1] : d0, sc[p], 0u);
-    }
-    rmax = __vimax3_s16x2(rmax, v[q * 4], v[q * 4 + 1]);
-    rmax = __vimax3_s16x2(rmax, v[q * 4 + 2], v[q * 4 + 3]);
-  }
-}
+// A pair of rows of the tensor-memory kernel (mpf_scan_kernel.cuh, row pairs:
+// cells and scores in units of 2^kCellShift).
 
-// The same with the node before the segment in the high half of `in_word`
-// (the lane before's pair 15, or a boundary-column word): no extraction.
-__device__ __forceinline__ void tile_row_regs_w(uint32_t (&v)[kPairs], uint32_t in_word,
+// Pair 0's diagonal: the node before the segment is in the high half of
+// in_word (the lane before's pair 15, or a boundary-column word).
+__device__ __forceinline__ uint32_t first_cell(uint32_t in_word, const uint32_t (&v)[kPairs]) {
+  return __byte_perm(in_word, v[kPairs - 1], 0x5432);
+}
+// First row: sums, not clamped.
+__device__ __forceinline__ void pair_row_first(uint32_t (&v)[kPairs], uint32_t in_word,
+                                               const uint32_t (&sc)[kPairs], uint32_t one) {
+  const uint32_t d0 = first_cell(in_word, v);
+#pragma unroll
+  for (int p = kPairs - 1; p >= 0; --p) v[p] = add_imad(p > 0 ? v[p - 1] : d0, sc[p], one);
+}
+// Second row: both rows' clamps, and the running maximum over both.
+__device__ __forceinline__ void pair_row_second(uint32_t (&v)[kPairs], uint32_t in_word,
                                                 const uint32_t (&sc)[kPairs], uint32_t &rmax) {
-  const uint32_t d0 = __byte_perm(in_word, v[kPairs - 1], 0x5432);
+  const uint32_t d0 = first_cell(in_word, v);
 #pragma unroll
-  for (int q = kChunks - 1; q >= 0; --q) {
-#pragma unroll
-    for (int e = 3; e >= 0; --e) {
-      const int p = q * 4 + e;
-      v[p] = __viaddmax_s16x2(p > 0 ? v[p - 1] : d0, sc[p], 0u);
-    }
-    rmax = __vimax3_s16x2(rmax, v[q * 4], v[q * 4 + 1]);
-    rmax = __vimax3_s16x2(rmax, v[q * 4 + 2], v[q * 4 + 3]);
+  for (int p = kPairs - 1; p >= 0; --p) {
+    const uint32_t prev = p > 0 ? v[p - 1] : d0;
+    const uint32_t u = __viaddmax_s16x2_relu(prev, sc[p], sc[p]);
+    rmax = __vimax3_s16x2(rmax, v[p], u);
+    v[p] = u;
   }
 }
 
-// MSV result of one sequence, by the whole warp: frow / fval, this lane's
-// first row with a cell above T and its largest cell there (kNone: none),
-// V this lane's largest cell.
+// MSV result of one sequence, by the whole warp: V, this lane's largest cell;
+// outcome, what the sweep decided (warp-uniform).
+enum Outcome { kExact, kOverflow, kRescore };
 __device__ __noinline__ void msv_finish(const ScanParams &sp, const QueryDesc &qd, uint32_t r, uint32_t len,
-                                        uint32_t orig, int lane, int b, int t, uint32_t frow, int fval, int V,
-                                        bool both) {
-  const int cap = 255 - qd.bias;
-  const uint32_t first = __reduce_min_sync(kAll, frow);
-  const int m = __reduce_max_sync(kAll, frow == first ? fval : -1);
+                                        uint32_t orig, int lane, int b, int t, int V, Outcome outcome, bool both) {
   V = __reduce_max_sync(kAll, V);
   if (both && lane == 0) {   // SSV from the same largest cell
     const int raw = min(V, 255);
@@ -139,7 +130,7 @@ __device__ __noinline__ void msv_finish(const ScanParams &sp, const QueryDesc &q
   // No cell rose above b: the best row maximum is the best single-cell
   // score of the residues (per-code maxima stored after the tiles).
   int g = -(1 << 20);
-  if (V == 0 && len > 0 && first == kNone) {
+  if (V == 0 && len > 0 && outcome == kExact) {
     const int16_t *smax =
         reinterpret_cast<const int16_t *>(reinterpret_cast<const uint8_t *>(qd.table) + qd.smax_off);
     const int mine = (int)__ldg(smax + lane);
@@ -157,20 +148,16 @@ __device__ __noinline__ void msv_finish(const ScanParams &sp, const QueryDesc &q
   if (lane != 0) return;
   int raw = 0, flag = 0;
   if (len > 0) {
-    if (first != kNone) {
-      if (b + m >= cap) {
-        raw = 255;
-        flag = 1;
-      } else if (first + 1 < len) {
-        // xB moves after this row: score the sequence exactly.
-        const uint32_t k = atomicAdd(qd.fallback_count, 1u);
-        if (MPF_DCHECK(sp.status, k < sp.n_seqs)) qd.fallback_ranks[k] = r;
-        return;
-      } else {
-        raw = max(0, b + V - qd.tec);
-      }
+    if (outcome == kOverflow) {
+      raw = 255;
+      flag = 1;
+    } else if (outcome == kRescore) {
+      // xB moves: score the sequence exactly.
+      const uint32_t k = atomicAdd(qd.fallback_count, 1u);
+      if (MPF_DCHECK(sp.status, k < sp.n_seqs)) qd.fallback_ranks[k] = r;
+      return;
     } else {
-      raw = V > 0 ? max(0, b + V - qd.tec) : max(0, b + g - qd.tec);
+      raw = max(0, b + (V > 0 ? V : g) - qd.tec);
     }
   }
   qd.raw[orig] = (uint8_t)raw;
@@ -312,7 +299,13 @@ __global__ void __launch_bounds__(kTileWarps * 32) tile_kernel(ScanParams sp) {
       }
     }
     if (MSV) {
-      if (active) msv_finish(sp, qd, r, len, orig, lane, b, tj, frow, fval, half_max(rmax), BOTH);
+      if (active) {
+        // The first row with a cell above T, and its maximum.
+        const uint32_t row = __reduce_min_sync(kAll, frow);
+        const int m = __reduce_max_sync(kAll, frow == row ? fval : -1);
+        const Outcome o = row == kNone ? kExact : b + m >= 255 - qd.bias ? kOverflow : row + 1 < len ? kRescore : kExact;
+        msv_finish(sp, qd, r, len, orig, lane, b, tj, half_max(rmax), o, BOTH);
+      }
       continue;
     }
     // R over the sequence: the largest half of any lane.
@@ -340,6 +333,11 @@ __global__ void __launch_bounds__(kTileWarps * 32) tile_kernel(ScanParams sp) {
 // from the tile in device memory.  One sequence per warp makes the residue
 // code of a row warp-uniform, so a row's 16 words are one tcgen05.ld, issued
 // a row ahead into the other of two register buffers.
+//
+// The sweep keeps the largest cell V only, which decides MSV as in the striped
+// held pass: at or above 255 - bias - b some row overflowed, at most T the
+// held rows are exact, in between the sequence goes to the fallback list.
+// Rows go in pairs (16 ALU instructions for 16 words instead of 24).
 template <bool MSV, bool BOTH>
 __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParams sp) {
   static_assert(MSV || !BOTH, "the both-filter sweep is the MSV sweep");
@@ -399,8 +397,6 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
     const int tj = qd.tjb ? (int)__ldg(qd.tjb + min(len, qd.n_tjb - 1u)) : qd.tjb_fixed;
     const int b = min(min(255, max(0, qd.base - (tj + qd.tbm))), 255 - qd.bias);
     const int T = min(qd.base + qd.tec - b, 255 - qd.bias - b - 1);
-    uint32_t frow = kNone;
-    int fval = -1;
     const int nt = (int)((qd.M + kTileNodes - 1) / kTileNodes);
     uint32_t rmax = 0;
     for (int t = 0; t < nt; ++t) {
@@ -444,30 +440,33 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
       // sequence; the load issued for the row after the last one takes any
       // code (only waited for).
       uint32_t TA[kPairs], TB[kPairs];
-      uint32_t word = len ? __ldg(sp.residues + w0) : 0u;
-      tm_ld<kPairs>(TA, tm_lane + (word & 31u) * (uint32_t)kPairs);
+      uint32_t word = (len ? __ldg(sp.residues + w0) : 0u) & 0x1f1f1f1fu;
+      tm_ld<kPairs>(TA, tm_lane + (word & 255u) * (uint32_t)kPairs);
+      uint32_t until_clear = 4 * kClearSteps;
       for (uint32_t i0 = 0; i0 < len; i0 += 4) {
-        const uint32_t nword = i0 + 4 < len ? __ldg(sp.residues + w0 + (i0 >> 2) + 1) : 0u;
+        // The next word, its codes masked to 0..31 (columns of the tile): a
+        // padding code's row is loaded but not used.
+        const uint32_t nword = (i0 + 4 < len ? __ldg(sp.residues + w0 + (i0 >> 2) + 1) : 0u) & 0x1f1f1f1fu;
         const uint4 c = cur;
         if (lane == 0 && !first) {
           cur = nxt;
           nxt = __ldcg(reinterpret_cast<const uint4 *>(cin) + (i0 >> 2) + 2);
         }
         const uint32_t cs[4] = {c.x, c.y, c.z, c.w};
-        uint32_t rq[4] = {0u, 0u, 0u, 0u};
         // One row: wait for its scores, issue the next row's load, update.
-        // The next row's code is masked to 0..31 (a column of the tile): in
-        // the sequence's last group of rows it may be a padding byte, whose
-        // load is only waited for.
         auto one_row = [&](const int u, uint32_t (&Tc)[kPairs], uint32_t (&Tn)[kPairs]) {
           tm_wait_ld<kPairs>(Tc);
-          MPF_DCHECK(sp.status, __byte_perm(word, 0u, 0x4440 + u) < 32u);
-          const uint32_t xn = (u < 3 ? __byte_perm(word, 0u, 0x4441 + u) : nword) & 31u;
+          const uint32_t xn = u < 3 ? __byte_perm(word, 0u, 0x4441 + u) : nword & 255u;
           tm_ld<kPairs>(Tn, tm_lane + xn * (uint32_t)kPairs);
           uint32_t in = __shfl_up_sync(kAll, v[kPairs - 1], 1);   // node 31 (high half), previous row
           if (lane == 0) in = cs[u];
-          tile_row_regs_w(v, in, Tc, MSV ? rq[u] : rmax);
-          if (write && lane == 31) cout[i0 + u + 1] = v[kPairs - 1];
+          if (u & 1)
+            pair_row_second(v, in, Tc, rmax);
+          else
+            pair_row_first(v, in, Tc, sp.one);
+          // The word handed on at the end of a group of rows carries no
+          // fraction past a clearing row of the next tile.
+          if (write && lane == 31) cout[i0 + u + 1] = u == 3 ? v[kPairs - 1] & kCellMask2 : v[kPairs - 1];
         };
         if (i0 + 4 <= len) {   // warp-uniform: four rows, no row test
           one_row(0, TA, TB);
@@ -475,45 +474,37 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
           one_row(2, TA, TB);
           one_row(3, TB, TA);
         } else {
+          const uint32_t left = len - i0;
+          one_row(0, TA, TB);
+          if (left > 1) one_row(1, TB, TA);
+          if (left > 2) one_row(2, TA, TB);
+          if (left != 2) {   // the last row has no second row to fold it
 #pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            if (i0 + u < len) {
-              if (u & 1)
-                one_row(u, TB, TA);
-              else
-                one_row(u, TA, TB);
-            }
+            for (int p = 0; p < kPairs; p += 2) rmax = __vimax3_s16x2(rmax, v[p], v[p + 1]);
           }
         }
         word = nword;
-        if (MSV) {
-          const uint32_t r4 = __vimax3_s16x2(rq[0], rq[1], __vimax_s16x2_relu(rq[2], rq[3]));
-          rmax = __vimax_s16x2_relu(rmax, r4);
-          if (i0 <= frow && half_max(r4) > T) {
+        until_clear -= 4;
+        if (until_clear == 0) {   // drop the sums' carries
+          until_clear = 4 * kClearSteps;
 #pragma unroll
-            for (int u = 3; u >= 0; --u) {
-              const int mu = half_max(rq[u]);
-              const uint32_t row = i0 + u;
-              if (mu > T && row < len) {
-                if (row < frow) {
-                  frow = row;
-                  fval = mu;
-                } else if (row == frow) {
-                  fval = max(fval, mu);
-                }
-              }
-            }
-          }
+          for (int p = 0; p < kPairs; ++p) v[p] &= kCellMask2;
         }
       }
+      tm_wait_ld<kPairs>(TB);
       tm_wait_ld<kPairs>(TA);   // the load issued after the last row
     }
+    const int V = half_max(rmax) >> kCellShift;
     if (MSV) {
-      if (active) msv_finish(sp, qd, r, len, orig, lane, b, tj, frow, fval, half_max(rmax), BOTH);
+      if (active) {
+        const int m = __reduce_max_sync(kAll, V);
+        const Outcome o = b + m >= 255 - qd.bias ? kOverflow : m > T ? kRescore : kExact;
+        msv_finish(sp, qd, r, len, orig, lane, b, tj, V, o, BOTH);
+      }
       continue;
     }
     int R = 0;
-    if (active) R = half_max(rmax);
+    if (active) R = V;
     R = __reduce_max_sync(kAll, R);
     if (active && lane == 0) {
       const int raw = min(R, 255);

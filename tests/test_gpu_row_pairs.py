@@ -30,15 +30,24 @@ def weak_profile(M, rng, K):
 @pytest.mark.parametrize("codes", [20, 21, 32])
 @pytest.mark.parametrize("lanes,words", CONFIGS)
 def test_long_weak_diagonals(lanes, words, codes):
+    rng = np.random.default_rng(1000 * lanes + words + codes)
+    check(2 * lanes * words - (words > 4) * int(rng.integers(0, 2 * lanes)), codes, rng, lanes, words)
+
+
+@pytest.mark.parametrize("M", [3073, 4100, 5000])
+def test_long_weak_diagonals_across_tiles(M):
+    """Models past the striped table: diagonals cross from tile to tile."""
+    check(M, 20, np.random.default_rng(M))
+
+
+def check(M, codes, rng, lanes=0, words=0):
     import torch
 
     import oracle
     from paper_1707_09683_gb300 import mpf
 
-    rng = np.random.default_rng(1000 * lanes + words + codes)
-    M = 2 * lanes * words - (words > 4) * int(rng.integers(0, 2 * lanes))
     p = weak_profile(M, rng, codes)
-    lengths = np.array([3, 119, 120, 121, 122, 240, 243, 1201, 0, 1, 777], dtype=np.uint32)
+    lengths = np.array([3, 119, 120, 121, 122, 240, 243, 1201, 0, 1, 777, 2, 1802], dtype=np.uint32)
     offsets = np.concatenate([[0], np.cumsum(lengths[:-1])]).astype(np.uint64)
     res = rng.integers(0, codes, size=int(lengths.sum())).astype(np.uint8)
     res[0] = codes - 1
@@ -46,7 +55,8 @@ def test_long_weak_diagonals(lanes, words, codes):
     ctx = mpf.Context(0)
     prof, db = mpf.Profile(ctx, p), mpf.Database(ctx, res, offsets, lengths)
     for filt in (mpf.MSV, mpf.SSV):
-        prof.set_config(filt, lanes, words)
+        if words:
+            prof.set_config(filt, lanes, words)
     want = [f(p, res, offsets, lengths) for f in (oracle.msv, oracle.ssv)]
     for filt, fn in ((mpf.MSV, mpf.msv_scan), (mpf.SSV, mpf.ssv_scan)):
         out = [torch.full((n,), 99, dtype=t, device="cuda") for t in (torch.uint8, torch.uint8, torch.float32)]
