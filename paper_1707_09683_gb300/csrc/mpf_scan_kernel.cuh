@@ -193,6 +193,14 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   constexpr bool kUnits = kSSV || kHeld;
   // SSV and held MSV with integer cells: rows in pairs (see the file comment).
   constexpr bool kPair = !kF16 && (kSSV || kHeld);
+  // Where a pair's cells join the running maximum, in two chains: row by row,
+  // two words per instruction, or both rows of a word with the second row,
+  // words alternating.  The first spreads the ALU work over both rows; long
+  // lanes are better off without its reads (GCUPS row by row / both rows,
+  // SSV, 60,000 sequences: 20 words 25,300 / 25,150, 26 25,080 / 24,330, 28
+  // 25,200 / 26,250, 38 25,420 / 26,140, 46 25,440 / 26,170; with one chain
+  // 23,300, 24,850, 25,060, 25,130, 22,810).
+  constexpr bool kFoldRows = H <= 26;
   const uint32_t one2 = 0x3c003c00u;   // (1.0, 1.0) as half2
   const uint32_t one = p.one;          // 1, opaque to the compiler (add_imad)
   extern __shared__ __align__(16) uint8_t smem[];
@@ -378,7 +386,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       uint32_t v[H];
 #pragma unroll
       for (int q = 0; q < H; ++q) v[q] = 0u;
-      uint32_t vacc = 0u;
+      uint32_t vacc = 0u, vacc2 = 0u;   // running maximum (vacc2: the other half of the row pairs' chain)
       int nsteps = 0;          // residue words of the rows
       bool busy = active;      // this group has rows to score
       uint32_t cur = 0u, ahead = 0u;   // the current residue word, and the next one as loaded
@@ -435,7 +443,10 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
                 v[q] = add_imad(prev, sc, one);
               } else {
                 const uint32_t u = __viaddmax_s16x2_relu(prev, sc, sc);
-                vacc = __vimax3_s16x2(vacc, v[q], u);
+                if constexpr (!kFoldRows) {
+                  uint32_t &acc = (q & 1) ? vacc2 : vacc;
+                  acc = __vimax3_s16x2(acc, v[q], u);
+                }
                 v[q] = u;
               }
             } else if (kF16)
@@ -447,8 +458,10 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
           };
           // Fold words q + 1 and q into the row / running maximum.
           auto fold = [&](const int q) {
-            if constexpr (kPair) return;   // folded with the cells of the pair's second row
-            if (kDirect)
+            if constexpr (kPair) {
+              uint32_t &acc = (rr & 1) == 0 ? vacc : vacc2;
+              if constexpr (kFoldRows) acc = __vimax3_s16x2(acc, v[q + 1], v[q]);
+            } else if (kDirect)
               rmax = __vimax3_u16x2(rmax, v[q + 1], v[q]);
             else
               vacc = __vimax3_u16x2(vacc, v[q + 1], v[q]);
@@ -607,6 +620,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
 
       // ---- finalise the G sequences -------------------------------------
       bool own = active && qvalid;   // this group writes its sequence's outputs
+      if constexpr (kPair) vacc = __vmaxs2(vacc, vacc2);
       int V = key_value<kF16>(group_max<LG>(half_max(vacc)));
       if (kUnits && __any_sync(kFull, split)) {
         // Of a split sequence's units the last one to finish goes on, with

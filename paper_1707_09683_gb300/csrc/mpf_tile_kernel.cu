@@ -94,21 +94,22 @@ __device__ __forceinline__ uint32_t first_cell(uint32_t in_word, const uint32_t 
 }
 // First row: sums, not clamped.
 __device__ __forceinline__ void pair_row_first(uint32_t (&v)[kPairs], uint32_t in_word,
-                                               const uint32_t (&sc)[kPairs], uint32_t one) {
+                                               const uint32_t (&sc)[kPairs], uint32_t &rmax, uint32_t one) {
   const uint32_t d0 = first_cell(in_word, v);
 #pragma unroll
-  for (int p = kPairs - 1; p >= 0; --p) v[p] = add_imad(p > 0 ? v[p - 1] : d0, sc[p], one);
+  for (int p = kPairs - 1; p >= 0; --p) {
+    v[p] = add_imad(p > 0 ? v[p - 1] : d0, sc[p], one);
+    if ((p & 1) == 0) rmax = __vimax3_s16x2(rmax, v[p + 1], v[p]);
+  }
 }
-// Second row: both rows' clamps, and the running maximum over both.
+// Second row: both rows' clamps.
 __device__ __forceinline__ void pair_row_second(uint32_t (&v)[kPairs], uint32_t in_word,
                                                 const uint32_t (&sc)[kPairs], uint32_t &rmax) {
   const uint32_t d0 = first_cell(in_word, v);
 #pragma unroll
   for (int p = kPairs - 1; p >= 0; --p) {
-    const uint32_t prev = p > 0 ? v[p - 1] : d0;
-    const uint32_t u = __viaddmax_s16x2_relu(prev, sc[p], sc[p]);
-    rmax = __vimax3_s16x2(rmax, v[p], u);
-    v[p] = u;
+    v[p] = __viaddmax_s16x2_relu(p > 0 ? v[p - 1] : d0, sc[p], sc[p]);
+    if ((p & 1) == 0) rmax = __vimax3_s16x2(rmax, v[p + 1], v[p]);
   }
 }
 
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
     const int b = min(min(255, max(0, qd.base - (tj + qd.tbm))), 255 - qd.bias);
     const int T = min(qd.base + qd.tec - b, 255 - qd.bias - b - 1);
     const int nt = (int)((qd.M + kTileNodes - 1) / kTileNodes);
-    uint32_t rmax = 0;
+    uint32_t rmax = 0, rmax2 = 0;   // running maxima over second and first rows of pairs
     for (int t = 0; t < nt; ++t) {
       // Every thread waited for its loads of the previous tile: order them
       // before this tile's TMEM writes.
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
           if (u & 1)
             pair_row_second(v, in, Tc, rmax);
           else
-            pair_row_first(v, in, Tc, sp.one);
+            pair_row_first(v, in, Tc, rmax2, sp.one);
           // The word handed on at the end of a group of rows carries no
           // fraction past a clearing row of the next tile.
           if (write && lane == 31) cout[i0 + u + 1] = u == 3 ? v[kPairs - 1] & kCellMask2 : v[kPairs - 1];
@@ -474,14 +475,9 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
           one_row(2, TA, TB);
           one_row(3, TB, TA);
         } else {
-          const uint32_t left = len - i0;
           one_row(0, TA, TB);
-          if (left > 1) one_row(1, TB, TA);
-          if (left > 2) one_row(2, TA, TB);
-          if (left != 2) {   // the last row has no second row to fold it
-#pragma unroll
-            for (int p = 0; p < kPairs; p += 2) rmax = __vimax3_s16x2(rmax, v[p], v[p + 1]);
-          }
+          if (i0 + 1 < len) one_row(1, TB, TA);
+          if (i0 + 2 < len) one_row(2, TA, TB);
         }
         word = nword;
         until_clear -= 4;
@@ -494,7 +490,7 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
       tm_wait_ld<kPairs>(TB);
       tm_wait_ld<kPairs>(TA);   // the load issued after the last row
     }
-    const int V = half_max(rmax) >> kCellShift;
+    const int V = half_max(__vmaxs2(rmax, rmax2)) >> kCellShift;
     if (MSV) {
       if (active) {
         const int m = __reduce_max_sync(kAll, V);
