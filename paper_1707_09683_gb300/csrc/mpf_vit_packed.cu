@@ -110,13 +110,21 @@ struct WarpPass {
 // word's seven planes are one tcgen05.ld.  In shared memory they took seven of
 // the eight L1 wavefronts per word (M = 2405: 82% of the pipe, 1,990 GCUPS).
 __host__ __device__ constexpr bool in_tmem(int qh, bool team) { return !team && qh > kVitPackRegQH; }
-// Threads per block at most (registers: 2 QH words of the row).
+// Threads per block at most (registers: 2 QH words of the row), and blocks
+// per SM that the registers must leave room for.  Without TMEM blocks are
+// small (a team, or four one-warp sequences), so that an SM whose sequences
+// of one launch have run out takes blocks of another, and a launch with few
+// sequences spreads them over the SMs (ms, 512-thread blocks / now: M = 100
+// on 10,000 sequences 1.06 / 0.91, M = 2405 on 2,000 1.83 / 1.65).
 __host__ __device__ constexpr int block_threads(int qh, bool team) {
-  return !in_tmem(qh, team) || qh <= kVitPack512QH ? kThreads : 384;
+  return team ? kThreads : !in_tmem(qh, team) ? 128 : qh <= kVitPack512QH ? kThreads : 384;
+}
+__host__ __device__ constexpr int block_min(int qh, bool team) {
+  return team || in_tmem(qh, team) ? 1 : qh <= 1 ? 8 : qh <= 2 ? 6 : qh <= 3 ? 5 : 4;
 }
 
 template <int QH, bool TEAM>
-__global__ void __launch_bounds__(block_threads(QH, TEAM), !TEAM && QH <= 2 ? 2 : 1)
+__global__ void __launch_bounds__(block_threads(QH, TEAM), block_min(QH, TEAM))
     viterbi_packed_kernel(VitParams p) {
   constexpr bool TM = in_tmem(QH, TEAM);
   __shared__ uint32_t s_tmem;
@@ -124,7 +132,7 @@ __global__ void __launch_bounds__(block_threads(QH, TEAM), !TEAM && QH <= 2 ? 2 
   __shared__ int s_max[4][kWarps];     // per team: largest M of a row (rows modulo 4)
   __shared__ WarpPass s_pass[kWarps];
   __shared__ uint32_t s_next[kWarps];
-  __shared__ int s_wn[3][kThreads];    // window sums of the later scan steps
+  __shared__ int s_wn[3][block_threads(QH, TEAM)];   // window sums of the later scan steps
   __shared__ int s_top[kWarps];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -554,7 +562,7 @@ int launch_viterbi_packed(const VitParams &p, VitPackShape s, int max_smem, int 
   if (p.n_queries == 0) return 0;
   const PackedFn fn = s.warps > 0 && s.warps <= kWarps ? packed_for(s) : nullptr;
   if (!fn) return 2;
-  const int threads = 32 * s.warps * (block_threads(s.qh, s.warps > 1) / 32 / s.warps);
+  const int threads = s.warps > 1 ? 32 * s.warps : block_threads(s.qh, false);
   // A block with its transitions in tensor memory takes all of the SM's
   // columns: it asks for more than half the shared memory, so that no second
   // block that does so is placed on the SM.  The match scores come through
@@ -567,7 +575,9 @@ int launch_viterbi_packed(const VitParams &p, VitPackShape s, int max_smem, int 
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, threads, smem) != cudaSuccess ||
       per_sm < 1 || (tm && per_sm != 1))
     return 1;
-  const int carve = (int)((size_t)per_sm * (smem + 9 * 1024) * 100 / (228 * 1024)) + 1;
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, (const void *)fn) != cudaSuccess) return 1;
+  const int carve = (int)((size_t)per_sm * (smem + a.sharedSizeBytes + 1024) * 100 / (228 * 1024)) + 1;
   if (cudaFuncSetAttribute((const void *)fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve) != cudaSuccess)
     return 1;
   VitParams q = p;
