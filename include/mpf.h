@@ -163,7 +163,8 @@ int mpf_profile_footprint(const mpf_profile *prof, int filter, uint32_t *smem_by
 /*
  * Cell arithmetic of a profile's scans for one filter.  Both give identical
  * results (the recurrences stay exact): MPF_ARITH_I16 updates two 16-bit
- * integer cells per DPX instruction on the integer pipe, MPF_ARITH_F16 holds
+ * integer cells per DPX instruction on the integer pipe (SSV and held MSV: of
+ * two rows, the first one's sums by integer multiply-adds), MPF_ARITH_F16 holds
  * the same integers as half-precision values and updates them with a fused
  * add-and-clamp on the FMA pipe.  MPF_ARITH_AUTO (default) is MPF_ARITH_I16:
  * no floating point in the cell updates.
@@ -177,7 +178,8 @@ int mpf_profile_set_arith(mpf_profile *prof, int filter, int arith);
  * it through the read-only cache).  Every striped kernel stages the table in
  * shared memory; with one sequence per warp (lanes 32, words >= 8) the
  * automatic choice also copies the first words of each lane's row (all of
- * them up to 14 words per lane, else 12) into the SM's tensor memory (TMEM,
+ * them up to 14 words per lane, else 12; up to 24, or 24, when every residue
+ * code of the database is below 20) into the SM's tensor memory (TMEM,
  * read by tcgen05.ld at about three times the shared-memory rate) and reads
  * those words from there.  For long models the tiled kernels' automatic
  * choice holds each 1,024-node tile in TMEM instead of shared memory (one
@@ -269,7 +271,9 @@ int mpf_scan_batch(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, in
  * Packed queries are sorted by words per lane; runs of them form sets where
  * a cost model in warp-words per row says a set pays, and each takes the
  * largest word count of its set (the added nodes score as padding: the
- * outputs do not change).
+ * outputs do not change).  Queries left over whose configuration was never
+ * set may share warps in mixed sets, each with as many lanes as its nodes
+ * need at the set's words per lane (databases whose codes are all below 20).
  *   mpf_plan_create:  arguments as mpf_scan_batch; raw/overflow/nat must be
  *                     device pointers (MPF_EINVAL otherwise).  The plan keeps
  *                     pointers to the profiles and database: they must outlive it.
@@ -285,8 +289,9 @@ int mpf_scan_batch(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, in
  *                     words per lane (0: tiled or long-model kernel), where
  *                     its table is read from (MPF_TABLE_SHARED or
  *                     MPF_TABLE_TENSOR), queries scored per warp and
- *                     sequence (1, or 32 / lanes when packed), its number
- *                     of queries and the filters it scores (1: MSV, 2: SSV,
+ *                     sequence (1, or 32 / lanes when packed; mixed sets:
+ *                     the most of any set, and 32 / that as the lanes), its
+ *                     number of queries and the filters it scores (1: MSV, 2: SSV,
  *                     3: both in one sweep).  Any output pointer may be NULL;
  *                     MPF_EINVAL for a NULL plan or i out of range.
  *   mpf_plan_pack_sets: the packed sets a plan forms among n queries of

@@ -64,6 +64,7 @@ def _units():
             units += [(src, f"mpf_inst_lg{lg}.o", [f"-DMPF_LG={lg}"]) for lg in INST_LANES]
             units.append((src, "mpf_inst_lg32_tm.o", ["-DMPF_LG=32", "-DMPF_TM=1"]))
             units += [(src, f"mpf_inst_qp{lg}_tm.o", [f"-DMPF_LG={lg}", "-DMPF_QP=1"]) for lg in QP_LANES]
+            units.append((src, "mpf_inst_mix.o", ["-DMPF_LG=32", "-DMPF_MIX=1"]))
             units.append((src, "mpf_inst_lg32_tmfew.o", ["-DMPF_LG=32", "-DMPF_TM=1", "-DMPF_FEW=1"]))
             units += [(src, f"mpf_inst_qp{lg}_tmfew.o", [f"-DMPF_LG={lg}", "-DMPF_QP=1", "-DMPF_FEW=1"])
                       for lg in QP_LANES]

@@ -186,6 +186,54 @@ int get_table(const mpf_profile *p, int lanes, int words, int fmt, DevTable *out
   return MPF_OK;
 }
 
+// Device copy of a profile's scores for a mixed set, on `lanes` lanes of
+// `words` words (striped as ever): row x, lane l, word q at ((x * lanes + l) *
+// words + q) * 4, then the 33 per-code best scores (TableGeom::smax_off).
+int get_mix_table(const mpf_profile *p, int lanes, int words, DevTable *out) {
+  std::lock_guard<std::mutex> lk(p->mu);
+  const auto key = std::make_tuple(lanes, words, (int)TABLE_I16_MIX);
+  auto it = p->tables.find(key);
+  if (it != p->tables.end()) {
+    *out = it->second;
+    return MPF_OK;
+  }
+  DevTable t;
+  t.geom = TableGeom{};
+  t.geom.smax_off = (uint32_t)(kTableRows * lanes * words * 4);
+  t.geom.table_bytes = (t.geom.smax_off + 80u + 15u) & ~15u;
+  std::vector<uint8_t> img(t.geom.table_bytes, 0);
+  int16_t *cell = reinterpret_cast<int16_t *>(img.data());
+  int16_t *smax = reinterpret_cast<int16_t *>(&img[t.geom.smax_off]);
+  const int M = p->M;
+  for (int x = 0; x < kTableRows; ++x) {
+    int m = kNegInf;
+    for (int k = 0; k < 2 * lanes * words; ++k) {
+      int s = kNegInf;
+      if (x < 32 && k < M) {
+        const int sv = p->bias - (x < p->K ? (int)p->cost[(size_t)x * M + k] : 255);
+        m = std::max(m, sv);
+        s = sv * (1 << kCellShift);
+      }
+      const int q = k % words, half = k / words % 2, l = k / words / 2;
+      cell[(((size_t)x * lanes + l) * words + q) * 2 + half] = (int16_t)s;
+    }
+    smax[x] = (int16_t)m;
+  }
+  mpf_ctx *ctx = p->ctx;
+  DeviceGuard dg(ctx->device);
+  MPF_CUDA(cudaMallocAsync((void **)&t.ptr, img.size(), ctx->util));
+  cudaError_t e = cudaMemcpyAsync(t.ptr, img.data(), img.size(), cudaMemcpyHostToDevice, ctx->util);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->util);
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    cudaFreeAsync(t.ptr, ctx->util);
+    return MPF_ECUDA;
+  }
+  p->tables[key] = t;
+  *out = t;
+  return MPF_OK;
+}
+
 // Device copy of a long profile's cost bytes in the long-model kernel's order:
 // residue row x, word w of lane l at (x * seg_words + w) * 32 + l, four nodes
 // (l * 4 * seg_words + 4w .. +3) per word; codes >= K and nodes past M cost 255.
@@ -323,6 +371,55 @@ bool use_tmem(const mpf_profile *p, int filter, int lanes, int words, int mode) 
          kernel_lg32_tm(words, mode) != nullptr;
 }
 
+// Mixed sets of queries whose one-query kernels take fewer than 32 lanes:
+// words per lane (0: none) and the sets, each a list of query numbers whose
+// lanes fit a warp.  Costs in warp-words per sequence row, fitted to measured
+// times (per 35.5 M residues, in units of 82 us: TMEM kernels of H words H +
+// 2.7; one-query kernels 5/4 of their warp-words, and 3): every built word
+// count is tried with first-fit decreasing, a set that costs no less than its
+// queries alone is dissolved.
+struct MixQuery {
+  int M, lanes, words;   // with its default configuration
+};
+std::pair<int, std::vector<std::vector<int>>> mix_sets(const std::vector<MixQuery> &qs) {
+  std::vector<int> order(qs.size());
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return qs[a].M > qs[b].M; });
+  auto alone = [&](int i) { return 1.25 * qs[i].words * qs[i].lanes / 32.0 + 3.0; };
+  std::pair<int, std::vector<std::vector<int>>> best(0, {});
+  double saved_best = 0;
+  for (int H = kMixWordsMin; H <= kMixWordsMax; H += 2) {
+    std::vector<std::vector<int>> sets;
+    std::vector<int> room;
+    for (int i : order) {
+      const int n = (qs[i].M + 2 * H - 1) / (2 * H);
+      if (n > 32) continue;
+      size_t s = 0;
+      while (s < sets.size() && room[s] < n) ++s;
+      if (s == sets.size()) {
+        sets.emplace_back();
+        room.push_back(32);
+      }
+      sets[s].push_back(i);
+      room[s] -= n;
+    }
+    double saved = 0;
+    std::vector<std::vector<int>> kept;
+    for (auto &s : sets) {
+      double a = -(H + 2.7);
+      for (int i : s) a += alone(i);
+      if (a <= 0 || s.size() < 2) continue;
+      saved += a;
+      kept.push_back(s);
+    }
+    if (saved > saved_best) {
+      saved_best = saved;
+      best = {H, kept};
+    }
+  }
+  return best;
+}
+
 // Packed sets of the candidates of one (lanes, mode), their word counts
 // ascending: runs [a, b) of consecutive queries; a run of two or more is a
 // set, padded to its largest word count, a run of one keeps its one-query
@@ -388,12 +485,18 @@ struct LaunchGroup {
   int shard_factor = 1;             // striped kernels: shards = factor x resident blocks
   uint32_t n_real = 0;              // queries of the group (n_queries less empty slots of packed sets)
   int qp = 1;                       // tensor-memory kernels: queries scored per warp and sequence
+  bool mix = false;                 // mixed sets: a warp's lanes dealt to the queries of a set
+  std::vector<uint32_t> mix_lanes;  //   32 words per set (ScanParams::mix_lanes)
+  int mix_queries = 0;              //   queries of the largest set
+  uint32_t *d_mix = nullptr;
   uint32_t qp_stride = 0;           //   and shared-memory bytes per staged table (qp > 1)
   // Split sequences (plan_split); n_long 0: none.
   uint32_t n_long = 0, n_long_units = 0, seg_rows = 0, seg_overlap = 0;
   uint32_t *d_units = nullptr;      // unit_rank, then unit_first
   std::shared_ptr<LaunchGroup> next;   // launched after this group on the same stream
 };
+
+constexpr int kMixedKey = 33;   // "queries per warp" of a mixed group's key
 
 struct mpf_plan {
   mpf_ctx *ctx = nullptr;
@@ -500,14 +603,17 @@ int configure_kernel(mpf_ctx *ctx, LaunchGroup *g) {
   // With the table in tensor memory: the few-codes kernel where the
   // database's codes allow it and it is built.
   g->fn = nullptr;
-  if (g->tm && g->tm_rows <= kTmFewCodes + 1)
+  if (g->mix)
+    g->fn = kernel_mix(g->words, g->mode);
+  else if (g->tm && g->tm_rows <= kTmFewCodes + 1)
     g->fn = g->qp > 1 ? kernel_qp_tmfew(g->lanes, g->words, g->mode) : kernel_lg32_tmfew(g->words, g->mode);
   if (!g->fn)
     g->fn = g->qp > 1 ? kernel_qp_tm(g->lanes, g->words, g->mode)
            : g->tm    ? kernel_lg32_tm(g->words, g->mode)
                       : kernel_for(g->lanes, g->words, g->mode);
   if (!g->fn) return MPF_EINVAL;
-  g->smem = g->qp > 1 ? (uint32_t)g->qp * g->qp_stride : (uint32_t)smem_need(g->lanes, g->words);
+  g->smem = g->mix ? 0u
+          : g->qp > 1 ? (uint32_t)g->qp * g->qp_stride : (uint32_t)smem_need(g->lanes, g->words);
   if (g->smem > (uint32_t)ctx->max_smem) return MPF_EUNSUPPORTED;
   // A block with the table in tensor memory takes all of the SM's TMEM
   // columns: ask for more than half the shared memory, so no second block of
@@ -524,10 +630,14 @@ int configure_kernel(mpf_ctx *ctx, LaunchGroup *g) {
   return MPF_OK;
 }
 
+// Queries, or sets of queries that share a warp.
+uint64_t group_sets(const LaunchGroup &g, size_t n_queries) {
+  return g.mix ? g.mix_lanes.size() / 32 : ((uint64_t)n_queries + g.qp - 1) / g.qp;
+}
+
 // Work of a launch group per residue, in words of a warp.
 double group_work(const LaunchGroup &g, const std::vector<QueryDesc> &queries) {
-  if (g.words)
-    return (double)((queries.size() + g.qp - 1) / g.qp) * g.words * (g.qp > 1 ? 1.0 : g.lanes / 32.0);
+  if (g.words) return (double)group_sets(g, queries.size()) * g.words * (g.qp > 1 ? 1.0 : g.lanes / 32.0);
   double w = 0;
   for (const QueryDesc &q : queries) w += q.M / 64.0;
   return w;
@@ -556,7 +666,7 @@ std::vector<uint32_t> plan_split(const mpf_db *db, double share, const std::vect
   for (const QueryDesc &q : queries) M = std::max(M, q.M);
   const uint64_t per_warp = g->qp > 1 ? 1 : 32 / (uint64_t)g->lanes;
   const uint64_t groups = (uint64_t)g->grid * (kBlockThreads / 32) * per_warp;
-  const uint64_t sets = ((uint64_t)queries.size() + g->qp - 1) / g->qp;
+  const uint64_t sets = group_sets(*g, queries.size());
   const uint64_t n_rows = (uint64_t)((double)(sets * db->n_residues / groups) / share);
   uint64_t S = std::max<uint64_t>({n_rows, M, kMinSegRows});
   const auto &len = db->longest;
@@ -612,7 +722,10 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     const mpf_profile *p;
     QueryDesc q;
     DevTable fb;
+    bool by_default;   // no configuration was set: it may join a mixed set
   };
+  std::map<int, std::vector<QpCand>> mix_cand;   // by mode
+  std::map<GroupKey, std::vector<uint32_t>> mix_lanes;
   std::map<std::pair<int, int>, std::vector<QpCand>> qp_cand;
   // One job per (query, kernel mode): MPF_MSV_SSV scores a query once for
   // both filters where it can (MODE_MSV_SSV, with the MSV settings), else
@@ -740,7 +853,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     if (n_q >= 2 && !ranks && !p->seg_words && lanes < 32 &&
         (mode == MODE_SSV || mode == MODE_MSV_HELD || mode == MODE_MSV_SSV) && words >= kTmMinWords &&
         p->table_mem[f] != MPF_TABLE_SHARED) {
-      qp_cand[std::make_pair(lanes, mode)].push_back(QpCand{words, sf, p, q, fb});
+      qp_cand[std::make_pair(lanes, mode)].push_back(QpCand{words, sf, p, q, fb, p->cfg_lanes[f] == 0});
       continue;
     }
     const GroupKey key(lanes, words, mode, tm, 1);
@@ -767,6 +880,10 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       const size_t a = r.first, b = r.second;
       const bool pack = b - a >= 2;
       const int H = v[b - 1].words;
+      if (!pack && v[a].by_default && db->code_end <= kTmFewCodes) {
+        mix_cand[mode].push_back(v[a]);
+        continue;
+      }
       const GroupKey key0(lanes, H, mode, 1, QP);
       for (size_t j = a; j < b; ++j) {
         QueryDesc q = v[j].q;
@@ -796,11 +913,61 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       }
     }
   }
+  // Mixed sets of the queries that are left over.  Their rescoring launch
+  // (one query per warp) takes 32 lanes, with the words that the longest needs.
+  for (auto &kv : mix_cand) {
+    const int mode = kv.first;
+    std::vector<QpCand> &v = kv.second;
+    std::vector<MixQuery> mq;
+    for (const QpCand &c : v) {
+      int lanes = 0, words = 0;
+      default_config(ctx, c.p->M, mode, &lanes, &words);
+      mq.push_back(MixQuery{c.p->M, lanes, words});
+    }
+    const auto mix = mix_sets(mq);
+    std::vector<bool> placed(v.size(), false);
+    int longest = 1;
+    for (const auto &set : mix.second)
+      for (int i : set) longest = std::max(longest, v[(size_t)i].p->M);
+    const int fb_words = std::max(4, (longest + 127) / 128 * 2);
+    const GroupKey key(32, mix.first, mode, 1, kMixedKey);
+    for (const auto &set : mix.second) {
+      std::vector<uint32_t> lane_of;
+      for (int i : set) {
+        QpCand &c = v[(size_t)i];
+        placed[(size_t)i] = true;
+        const int n = (c.p->M + 2 * mix.first - 1) / (2 * mix.first);
+        DevTable t;
+        int rc = get_mix_table(c.p, n, mix.first, &t);
+        if (rc == MPF_OK && mode != MODE_SSV) rc = get_table(c.p, 32, fb_words, TABLE_I16, &c.fb);
+        if (rc) {
+          plan_free(pl);
+          return rc;
+        }
+        set_table(c.q, t);
+        for (int l = 0; l < n; ++l)
+          lane_of.push_back((uint32_t)byconf[key].size() | (uint32_t)l << 16 | (uint32_t)n << 24);
+        byconf[key].push_back(c.q);
+        if (mode != MODE_SSV) fb_table[key].push_back(c.fb);
+        group_shards[key] = std::max(group_shards[key], c.sf);
+      }
+      lane_of.resize(32, 0u);
+      auto &ml = mix_lanes[key];
+      ml.insert(ml.end(), lane_of.begin(), lane_of.end());
+    }
+    for (size_t i = 0; i < v.size(); ++i) {
+      if (placed[i]) continue;
+      const GroupKey alone(mq[i].lanes, mq[i].words, mode, 0, 1);
+      byconf[alone].push_back(v[i].q);
+      if (mode != MODE_SSV) fb_table[alone].push_back(v[i].fb);
+      group_shards[alone] = std::max(group_shards[alone], v[i].sf);
+    }
+  }
   DeviceGuard dg(ctx->device);
   // Byte offsets of a group's parts in the plan's device memory: of the
   // uploaded part, and of the rest.
   struct Parts {
-    size_t desc = 0, fb_desc = 0, unit_tables = 0, zero = 0, fb_ranks = 0, unit_max = 0, col = 0;
+    size_t desc = 0, fb_desc = 0, unit_tables = 0, mix = 0, zero = 0, fb_ranks = 0, unit_max = 0, col = 0;
     std::vector<uint32_t> units;
   };
   struct Layout {
@@ -817,7 +984,9 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     LaunchGroup g;
     g.lanes = std::get<0>(kv.first);
     g.words = std::get<1>(kv.first);
-    g.qp = std::get<4>(kv.first);
+    g.mix = std::get<4>(kv.first) == kMixedKey;
+    if (g.mix) g.mix_lanes = mix_lanes[kv.first];
+    g.qp = g.mix ? 1 : std::get<4>(kv.first);
     work += group_work(g, kv.second);
   }
   for (auto &kv : byconf) {
@@ -826,7 +995,16 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     g.words = std::get<1>(kv.first);
     g.mode = std::get<2>(kv.first);
     g.tm = std::get<3>(kv.first) != 0;
-    g.qp = std::get<4>(kv.first);
+    g.mix = std::get<4>(kv.first) == kMixedKey;
+    if (g.mix) {
+      g.mix_lanes = mix_lanes[kv.first];
+      for (size_t i = 0; i < g.mix_lanes.size(); i += 32) {
+        int n = 0;
+        for (size_t l = i; l < i + 32; ++l) n += (g.mix_lanes[l] >> 24) && !(g.mix_lanes[l] >> 16 & 0xff);
+        g.mix_queries = std::max(g.mix_queries, n);
+      }
+    }
+    g.qp = g.mix ? 1 : std::get<4>(kv.first);
     if (g.qp > 1) g.qp_stride = packed_table_stride(g.lanes, g.words);
     g.shard_factor = group_shards[kv.first];
     for (const QueryDesc &qd : kv.second) g.long_words = std::max(g.long_words, qd.seg_words);
@@ -864,7 +1042,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       // 132-260).
       nx->mode = held ? MODE_MSV_FAST : MODE_LONG_MSV;
       nx->lanes = g.lanes;
-      nx->words = g.words;
+      nx->words = g.mix ? fb_table[kv.first][0].geom.words : g.words;
       nx->n_codes = db->n_codes;
       nx->n_long = g.n_long;
       nx->n_long_units = g.n_long_units;
@@ -889,6 +1067,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     pt.desc = up.take(sizeof(QueryDesc) * nq);
     pt.fb_desc = up.take(fallback ? sizeof(QueryDesc) * g.next->n_queries : 0);
     pt.unit_tables = up.take(4 * pt.units.size());
+    pt.mix = up.take(4 * g.mix_lanes.size());
     g.zero_words = 2 + (fallback ? nq : 0) + nq * g.n_long;
     pt.zero = rest.take(4 * g.zero_words);
     pt.fb_ranks = rest.take(fallback ? 4 * nq * ns : 0);
@@ -915,6 +1094,8 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       g.d_counter = g.d_zero = zero;
       g.d_col = g.col_bytes ? scratch + pt.col : nullptr;
       g.d_units = reinterpret_cast<uint32_t *>(base + pt.unit_tables);
+      g.d_mix = reinterpret_cast<uint32_t *>(base + pt.mix);
+      if (g.mix) memcpy(&host[pt.mix], g.mix_lanes.data(), 4 * g.mix_lanes.size());
       if (!pt.units.empty()) memcpy(&host[pt.unit_tables], pt.units.data(), 4 * pt.units.size());
       std::vector<QueryDesc> fq;
       for (size_t i = 0; i < nq; ++i) {
@@ -1003,7 +1184,9 @@ int enqueue_group(const mpf_db *db, mpf_ctx *ctx, LaunchGroup &g, cudaStream_t s
   sp.seg_overlap = g.seg_overlap;
   sp.unit_rank = g.d_units;
   sp.unit_first = g.d_units + g.n_long_units;
-  const uint64_t n_items = ((uint64_t)g.n_queries + (uint64_t)g.qp - 1) / (uint64_t)g.qp * g.n_shards;
+  sp.n_sets = (uint32_t)(g.mix_lanes.size() / 32);
+  sp.mix_lanes = g.d_mix;
+  const uint64_t n_items = group_sets(g, g.n_queries) * g.n_shards;
   const int grid = (int)std::min<uint64_t>((uint64_t)g.grid, n_items);
   g.fn<<<grid, g.threads, g.smem, st>>>(sp);
   MPF_CUDA(cudaGetLastError());
@@ -1530,10 +1713,10 @@ int mpf_plan_group_info(const mpf_plan *plan, int i, int *lanes, int *words, int
                         int *queries_per_warp, int *n_queries, int *filters) {
   if (!plan || i < 0 || (size_t)i >= plan->groups.size()) return MPF_EINVAL;
   const LaunchGroup &g = plan->groups[(size_t)i];
-  if (lanes) *lanes = g.lanes;
+  if (lanes) *lanes = g.mix ? std::max(1, 32 / g.mix_queries) : g.lanes;
   if (words) *words = g.words;
   if (table_memory) *table_memory = g.tm ? MPF_TABLE_TENSOR : MPF_TABLE_SHARED;
-  if (queries_per_warp) *queries_per_warp = g.qp;
+  if (queries_per_warp) *queries_per_warp = g.mix ? g.mix_queries : g.qp;
   if (n_queries) *n_queries = (int)g.n_real;
   if (filters) {
     switch (g.mode) {

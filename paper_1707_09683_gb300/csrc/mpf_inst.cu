@@ -11,6 +11,7 @@
 // Either with -DMPF_FEW=1 builds the variants for databases of few residue
 // codes (kernel_lg32_tmfew(), kernel_qp_tmfew_lg<lanes>(): those three modes,
 // from 16 words on; shorter lanes fit tensor memory whole with every code).
+// -DMPF_LG=32 -DMPF_MIX=1 builds kernel_mix(): the same modes for mixed sets.
 #include "mpf_scan_kernel.cuh"
 
 #ifndef MPF_LG
@@ -28,7 +29,24 @@
 
 namespace mpf {
 
-#if defined(MPF_QP) || (defined(MPF_TM) && defined(MPF_FEW))
+#if defined(MPF_MIX)
+
+#define MPF_CASE(W)                                                                              \
+  case W:                                                                                        \
+    if (mode == MODE_SSV) return scan_kernel<32, W, MODE_SSV, TM_FEW, 1, true>;                  \
+    if (mode == MODE_MSV_HELD) return scan_kernel<32, W, MODE_MSV_HELD, TM_FEW, 1, true>;        \
+    if (mode == MODE_MSV_SSV) return scan_kernel<32, W, MODE_MSV_SSV, TM_FEW, 1, true>;          \
+    return nullptr;
+
+KernelFn kernel_mix(int words, int mode) {
+  switch (words) {
+    MPF_CASE(14) MPF_CASE(16) MPF_CASE(18) MPF_CASE(20) MPF_CASE(22) MPF_CASE(24)
+    default:
+      return nullptr;
+  }
+}
+
+#elif defined(MPF_QP) || (defined(MPF_TM) && defined(MPF_FEW))
 
 #ifdef MPF_QP
 constexpr int kQueries = 32 / MPF_LG;

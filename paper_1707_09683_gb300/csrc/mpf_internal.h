@@ -97,7 +97,7 @@ __host__ __device__ constexpr int tm_words(int words, int tm) {
 // Score-table formats: signed 16-bit integers, or the same integers as fp16.
 // TABLE_I16_PACKED: integer scores in the packed geometry (one copy of each
 // region; the tables of the queries that share a warp's sequence).
-enum TableFormat : int { TABLE_I16 = 0, TABLE_F16 = 1, TABLE_I16_PACKED = 16 };
+enum TableFormat : int { TABLE_I16 = 0, TABLE_F16 = 1, TABLE_I16_PACKED = 16, TABLE_I16_MIX = 17 };
 inline int table_format(int mode) {
   return (mode == MODE_SSV_F16 || mode == MODE_MSV_FAST_F16 || mode == MODE_MSV_HELD_F16) ? TABLE_F16
                                                                                            : TABLE_I16;
@@ -161,6 +161,8 @@ struct ScanParams {
   // seg_overlap rows before), then the other ranks whole.
   uint32_t n_units, n_long, n_long_units, seg_rows, seg_overlap;
   const uint32_t *unit_rank, *unit_first;
+  uint32_t n_sets;            // mixed sets: their number, and 32 words per set (query | lane of its
+  const uint32_t *mix_lanes;  //   group << 16 | lanes of the group << 24; 0 lanes: none)
   uint32_t tm_rows;           // TM_FEW kernels: TMEM rows, the database's codes and the padding code
   uint32_t one;               // 1 (striped kernels: see add_imad)
   uint32_t qp_table_stride;   // striped kernels with several queries per warp: bytes per staged table
@@ -318,6 +320,9 @@ KernelFn kernel_for(int lanes, int words, int mode);
 // counts on where it differs), or nullptr if not built.
 KernelFn kernel_lg32_tm(int words, int mode);
 KernelFn kernel_lg32_tmfew(int words, int mode);
+// Mixed sets (few codes, every word in tensor memory).
+KernelFn kernel_mix(int words, int mode);
+constexpr int kMixWordsMin = 14, kMixWordsMax = 24;
 // Tensor-memory variants that score one sequence against 32 / lanes queries
 // per warp (lanes 1 to 16), or nullptr if not built.
 KernelFn kernel_qp_tm(int lanes, int words, int mode);

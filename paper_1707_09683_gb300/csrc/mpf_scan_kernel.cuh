@@ -53,6 +53,15 @@
 // (GB300, clock64, 16 words per lane, table in registers): 52.7 words per
 // clock and SM against 42.4 for two rows of add-then-max.
 //
+// Mixed sets (MIX).  A warp's lanes are dealt to several queries of any
+// length, each with as many lanes as its nodes fill at H words per lane, and
+// all score the warp's one sequence: the rows of every lane come from tensor
+// memory at one residue's column, as for one query on 32 lanes.  A batch's
+// shorter queries otherwise run kernels whose groups read different residues
+// from shared memory, at half the rate (GCUPS alone, 100,000 sequences: M =
+// 48 / 100 / 200 / 400 / 800 5,570 / 8,350 / 12,430 / 16,280 / 17,480; a set
+// of 48, 200, 400 and 800 on 24 words 24,890).
+//
 // Segments.  A path of the SSV recurrence (and of held MSV, the same cells)
 // visits at most M rows, so the largest cell of rows a .. b - 1 is known from
 // a zero row M rows before a: a long sequence splits into segments of
@@ -168,12 +177,24 @@ __device__ __forceinline__ uint32_t pack2_half(int v) {
   return (h << 16) | h;
 }
 
-template <int LG, int H, int MODE, int TM = TM_NONE, int QP = 1>
+// group_max for groups of any width side by side: this lane is lane gl of its
+// group of `width` (every lane gets its group's maximum).
+__device__ __forceinline__ int mixed_max(int v, int lane, int gl, int width) {
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int y = __shfl_down_sync(kFull, v, off);
+    if (gl + off < width) v = max(v, y);
+  }
+  return __shfl_sync(kFull, v, lane - gl);
+}
+
+template <int LG, int H, int MODE, int TM = TM_NONE, int QP = 1, bool MIX = false>
 __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   static_assert((H % 4 == 0 || H % 4 == 2) && H >= 4 && H <= kMaxWords, "words per lane");
   static_assert(!TM || ((LG == 32 || QP * LG == 32) && H >= kTmMinWords && MODE != MODE_MSV_DIRECT),
                 "tensor-memory variant");
   static_assert(QP == 1 || (TM && QP * LG == 32), "queries per warp");
+  static_assert(!MIX || (TM == TM_FEW && LG == 32 && QP == 1 && tm_words(H, TM) == H), "mixed sets");
   constexpr int HT = tm_words(H, TM);   // words per lane from TMEM
   static_assert(HT == H || HT % 4 == 0, "shared-memory words start on a chunk");
   constexpr int Q = H / 4;               // full 4-word chunks per lane and row
@@ -208,20 +229,22 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   __shared__ uint32_t s_tmem;
 
   const int lane = threadIdx.x & 31;
-  const int gl = lane & (LG - 1);
+  int gl = lane & (LG - 1), width = LG;   // lane of the group, its lanes (mixed sets: per item)
   const int grp = lane / LG;
   // Byte selector of the diagonal shift: bytes 2, 3 of the lane before's last
   // word, then bytes 0, 1 of this lane's.  With integer cells (0 .. 32767)
   // the group's first lane takes the sign copies of its own byte 1, which
   // are zero; fp16 cells zero it with a select instead.
-  const uint32_t shift_sel = (LG > 1 && gl != 0) ? 0x5432u : 0x54ddu;
+  uint32_t shift_sel = (LG > 1 && gl != 0) ? 0x5432u : 0x54ddu;
   // QP > 1: the 32 / LG groups of a warp score one sequence against QP
   // queries (the QP consecutive queries of a work item), so every lane of
   // the warp reads the same residue and the TMEM column of a row is uniform.
   // Every lane of a warp follows the same sequence: a warp reduction (whose
   // result is uniform) hands each residue word to the rows.
   constexpr bool kUniform = TM != TM_NONE;
-  const uint32_t n_items = (p.n_queries + QP - 1) / QP * p.n_shards;
+  // Mixed sets: item i scores set i / n_shards, whose lanes belong to queries
+  // as p.mix_lanes says (query, lane of its group, width; width 0: no query).
+  const uint32_t n_items = (MIX ? p.n_sets : (p.n_queries + QP - 1) / QP) * p.n_shards;
   const int warp = (int)(threadIdx.x >> 5);
   uint32_t tm_lane = 0;   // TMEM address of this warp's lane quarter, column 0
   if constexpr (TM) {
@@ -243,8 +266,16 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
     const uint32_t item = s_item;
     if (item >= n_items) break;
     const uint32_t shard = item % p.n_shards;
-    const uint32_t qbase = item / p.n_shards * QP;
-    const uint32_t qi = qbase + (QP > 1 ? (uint32_t)grp : 0u);
+    uint32_t qbase = item / p.n_shards * QP;
+    uint32_t qi = qbase + (QP > 1 ? (uint32_t)grp : 0u);
+    if constexpr (MIX) {
+      const uint32_t m = __ldg(p.mix_lanes + qbase * 32 + lane);
+      qbase = __ldg(p.mix_lanes + qbase * 32) & 0xffffu;   // lane 0 always has a query
+      width = (int)(m >> 24);
+      gl = (int)((m >> 16) & 0xffu);
+      qi = width ? m & 0xffffu : p.n_queries;
+      shift_sel = gl != 0 ? 0x5432u : 0x54ddu;
+    }
     // QP > 1: a set may have empty slots (descriptors without a table, after
     // its queries), and the last item fewer queries.
     const bool qvalid = qi < p.n_queries && (QP == 1 || p.queries[qi].table != nullptr);
@@ -269,7 +300,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
     // Stage the striped table(s) (16-byte vector copies, coalesced); with
     // QP > 1 query g's table at g * tstride.
 #pragma unroll 1
-    for (int g = 0; g < QP; ++g) {
+    for (int g = 0; g < (MIX ? 0 : QP); ++g) {
       if (qbase + (uint32_t)g >= p.n_queries) break;
       const QueryDesc *qg = p.queries + qbase + g;
       if (!qg->table) continue;
@@ -290,7 +321,21 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       // Copy the first HT words of every lane's row of every code from the
       // staged table into tensor memory: warp q < 4 writes lane quarter q.
       tm_fence_after();
-      if (warp < 4) {
+      if constexpr (MIX) {
+        // Straight from device memory, rows dealt to the warps of a quarter.
+        const uint2 *src = reinterpret_cast<const uint2 *>(qd->table) + (size_t)gl * (H / 2);
+        for (uint32_t row = warp >> 2; row <= tm_pad; row += kBlockThreads / 128) {
+          const uint32_t x = row == tm_pad ? (uint32_t)kPadCode : row;
+          const uint2 *s2 = src + (size_t)x * (uint32_t)width * (H / 2);
+          const uint32_t col = tm_lane + row * (uint32_t)HT;
+          uint2 w[H / 2];
+#pragma unroll
+          for (int j = 0; j < H / 2; ++j) w[j] = width ? __ldg(s2 + j) : make_uint2(0xc000c000u, 0xc000c000u);
+#pragma unroll
+          for (int j = 0; j < H / 2; ++j) tm_st2(col + 2 * j, w[j].x, w[j].y);
+        }
+        tm_wait_st();
+      } else if (warp < 4) {
         for (uint32_t row = 0; row <= tm_pad; ++row) {
           const uint32_t col = tm_lane + row * (uint32_t)HT;
           const uint32_t x = row == tm_pad ? (uint32_t)kPadCode : row;
@@ -322,7 +367,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
     float *out_nat = qd->nat;
     const uint32_t row_bytes = qd->row_bytes;
     const uint32_t tail_row_bytes = qd->tail_row_bytes;
-    const int16_t *smax = reinterpret_cast<const int16_t *>(tbl_base + qd->smax_off);
+    const int16_t *smax = reinterpret_cast<const int16_t *>(
+        (MIX ? reinterpret_cast<const uint8_t *>(qd->table) : tbl_base) + qd->smax_off);
+    auto gmax = [&](int x) { return MIX ? mixed_max(x, lane, gl, width) : group_max<LG>(x); };
     const uint32_t *ranks = qd->ranks;
     const uint64_t n_sel = ranks ? (uint64_t)*qd->n_ranks : (uint64_t)p.n_units;
 
@@ -621,7 +668,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       // ---- finalise the G sequences -------------------------------------
       bool own = active && qvalid;   // this group writes its sequence's outputs
       if constexpr (kPair) vacc = __vmaxs2(vacc, vacc2);
-      int V = key_value<kF16>(group_max<LG>(half_max(vacc)));
+      int V = key_value<kF16>(gmax(half_max(vacc)));
       if (kUnits && __any_sync(kFull, split)) {
         // Of a split sequence's units the last one to finish goes on, with
         // the largest cell of all of them.
@@ -639,8 +686,8 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         last = __shfl_sync(kFull, last, lane - gl);
         own = own && last;
         if (split && own)
-          for (uint32_t u = gl; u < n; u += LG) V = max(V, __ldcg(qd->unit_max + first + u));
-        V = group_max<LG>(V);
+          for (uint32_t u = gl; u < n; u += (uint32_t)width) V = max(V, __ldcg(qd->unit_max + first + u));
+        V = gmax(V);
       }
       if (kFast || kHeld) {
         // A sequence whose cells never rose above the begin score: its best
@@ -648,7 +695,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         const bool rescue = own && !done && !exact && V == 0 && len > 0;
         int g = INT_MIN / 2;
         if (rescue) {
-          for (int w = gl; w < (len + 3) >> 2; w += LG) {
+          for (int w = gl; w < (len + 3) >> 2; w += width) {
             const uint32_t word = __ldg(p.residues + wstart + (uint32_t)w);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -656,7 +703,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
                 g = max(g, (int)smax[(word >> (8 * i)) & 0xffu]);
           }
         }
-        g = group_max<LG>(g);
+        g = gmax(g);
         if (kBoth && own && gl == 0) {
           // SSV (Alg. 7) from the same largest cell: with b held the MSV
           // cells minus b are exactly the SSV cells.
