@@ -496,6 +496,13 @@ struct LaunchGroup {
   std::shared_ptr<LaunchGroup> next;   // launched after this group on the same stream
 };
 
+// The rescoring launch on 32 lanes per sequence: words per lane for the
+// longest of its queries.  It takes the queries with at most kRescoreWidePerSm
+// sequences per SM listed, where a row's latency counts; with more, the
+// launch with the query's own lanes scores more sequences per warp.
+int rescore_words(int longest) { return std::max(4, (longest + 127) / 128 * 2); }
+constexpr int kRescoreWidePerSm = 48;
+
 constexpr int kMixedKey = 33;   // "queries per warp" of a mixed group's key
 
 struct mpf_plan {
@@ -712,7 +719,11 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
   // per warp).
   using GroupKey = std::tuple<int, int, int, int, int>;
   std::map<GroupKey, std::vector<QueryDesc>> byconf;
-  std::map<GroupKey, std::vector<DevTable>> fb_table;   // tables of the exact rescoring launch
+  struct Rescore {           // table of a query's exact rescoring launch, and its profile
+    DevTable t;
+    const mpf_profile *p;
+  };
+  std::map<GroupKey, std::vector<Rescore>> fb_table;
   std::map<GroupKey, std::vector<uint32_t>> fb_seg_words;
   std::map<GroupKey, int> group_shards;   // largest shard factor of a group's profiles
   // Queries that may share a warp's sequence with others (fewer than 32
@@ -785,7 +796,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
         }
         DevTable lt_t{};
         lt_t.ptr = reinterpret_cast<uint4 *>(const_cast<uint8_t *>(lt));
-        fb_table[GroupKey(lanes, words, mode, ttm, 1)].push_back(lt_t);
+        fb_table[GroupKey(lanes, words, mode, ttm, 1)].push_back(Rescore{lt_t, p});
         fb_seg_words[GroupKey(lanes, words, mode, ttm, 1)].push_back((uint32_t)p->seg_words);
       }
     } else if (p->seg_words) {
@@ -858,7 +869,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     }
     const GroupKey key(lanes, words, mode, tm, 1);
     byconf[key].push_back(q);
-    if (fb.ptr) fb_table[key].push_back(fb);
+    if (fb.ptr) fb_table[key].push_back(Rescore{fb, p});
     group_shards[key] = std::max(group_shards[key], sf);
   }
   // Several queries per warp: 32 / lanes queries of one (lanes, mode) score
@@ -900,7 +911,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
         }
         const GroupKey key = pack ? key0 : GroupKey(lanes, v[j].words, mode, 0, 1);
         byconf[key].push_back(q);
-        if (mode != MODE_SSV) fb_table[key].push_back(fb);
+        if (mode != MODE_SSV) fb_table[key].push_back(Rescore{fb, v[j].p});
         group_shards[key] = std::max(group_shards[key], v[j].sf);
       }
       if (pack) {
@@ -908,7 +919,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
         memset(&empty, 0, sizeof(empty));
         for (size_t j = b - a; j < (size_t)QP; ++j) {
           byconf[key0].push_back(empty);
-          if (mode != MODE_SSV) fb_table[key0].push_back(DevTable{});
+          if (mode != MODE_SSV) fb_table[key0].push_back(Rescore{});
         }
       }
     }
@@ -929,7 +940,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     int longest = 1;
     for (const auto &set : mix.second)
       for (int i : set) longest = std::max(longest, v[(size_t)i].p->M);
-    const int fb_words = std::max(4, (longest + 127) / 128 * 2);
+    const int fb_words = rescore_words(longest);
     const GroupKey key(32, mix.first, mode, 1, kMixedKey);
     for (const auto &set : mix.second) {
       std::vector<uint32_t> lane_of;
@@ -948,7 +959,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
         for (int l = 0; l < n; ++l)
           lane_of.push_back((uint32_t)byconf[key].size() | (uint32_t)l << 16 | (uint32_t)n << 24);
         byconf[key].push_back(c.q);
-        if (mode != MODE_SSV) fb_table[key].push_back(c.fb);
+        if (mode != MODE_SSV) fb_table[key].push_back(Rescore{c.fb, c.p});
         group_shards[key] = std::max(group_shards[key], c.sf);
       }
       lane_of.resize(32, 0u);
@@ -959,7 +970,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       if (placed[i]) continue;
       const GroupKey alone(mq[i].lanes, mq[i].words, mode, 0, 1);
       byconf[alone].push_back(v[i].q);
-      if (mode != MODE_SSV) fb_table[alone].push_back(v[i].fb);
+      if (mode != MODE_SSV) fb_table[alone].push_back(Rescore{v[i].fb, v[i].p});
       group_shards[alone] = std::max(group_shards[alone], v[i].sf);
     }
   }
@@ -969,6 +980,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
   struct Parts {
     size_t desc = 0, fb_desc = 0, unit_tables = 0, mix = 0, zero = 0, fb_ranks = 0, unit_max = 0, col = 0;
     std::vector<uint32_t> units;
+    std::vector<DevTable> wide;   // per query: table of the rescoring launch on 32 lanes
   };
   struct Layout {
     size_t bytes = 0;
@@ -1042,7 +1054,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       // 132-260).
       nx->mode = held ? MODE_MSV_FAST : MODE_LONG_MSV;
       nx->lanes = g.lanes;
-      nx->words = g.mix ? fb_table[kv.first][0].geom.words : g.words;
+      nx->words = g.mix ? fb_table[kv.first][0].t.geom.words : g.words;
       nx->n_codes = db->n_codes;
       nx->n_long = g.n_long;
       nx->n_long_units = g.n_long_units;
@@ -1055,20 +1067,36 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       }
       nx->n_real = nx->n_queries;
       int rc2 = configure_kernel(ctx, nx.get());
+      if (rc2 == MPF_OK && held && g.lanes < 32) {
+        // Queries with few listed sequences take 32 lanes for each instead.
+        auto wide = std::make_shared<LaunchGroup>(*nx);
+        int longest = 1;
+        for (const QueryDesc &qd : kv.second) longest = std::max(longest, (int)qd.M);
+        wide->lanes = 32;
+        wide->words = rescore_words(longest);
+        pt.wide.resize(nq);
+        for (size_t i = 0; i < nq && rc2 == MPF_OK; ++i)
+          if (kv.second[i].table)
+            rc2 = get_table(fb_table[kv.first][i].p, 32, wide->words, TABLE_I16, &pt.wide[i]);
+        if (rc2 == MPF_OK) rc2 = configure_kernel(ctx, wide.get());
+        wide->next = nx;
+        g.next = wide;
+      } else {
+        g.next = nx;
+      }
       if (rc2) {
         plan_free(pl);
         return rc2;
       }
-      g.next = nx;
     }
     // What is uploaded (descriptors, unit tables), what is zeroed before each
     // launch (the work counters of the group and its fallback launch, the
     // fallback counts, the finished units), and scratch.
     pt.desc = up.take(sizeof(QueryDesc) * nq);
-    pt.fb_desc = up.take(fallback ? sizeof(QueryDesc) * g.next->n_queries : 0);
+    pt.fb_desc = up.take(fallback ? sizeof(QueryDesc) * g.next->n_queries * (g.next->next ? 2 : 1) : 0);
     pt.unit_tables = up.take(4 * pt.units.size());
     pt.mix = up.take(4 * g.mix_lanes.size());
-    g.zero_words = 2 + (fallback ? nq : 0) + nq * g.n_long;
+    g.zero_words = 3 + (fallback ? nq : 0) + nq * g.n_long;
     pt.zero = rest.take(4 * g.zero_words);
     pt.fb_ranks = rest.take(fallback ? 4 * nq * ns : 0);
     pt.unit_max = rest.take(4 * nq * g.n_long_units);
@@ -1087,7 +1115,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       const Parts &pt = parts[gi++];
       const size_t nq = kv.second.size(), ns = std::max<uint64_t>(db->n_seqs, 1);
       uint32_t *zero = reinterpret_cast<uint32_t *>(scratch + pt.zero);
-      uint32_t *fb_count = zero + 2, *unit_done = fb_count + (g.next ? nq : 0);
+      uint32_t *fb_count = zero + 3, *unit_done = fb_count + (g.next ? nq : 0);
       uint32_t *fb_ranks = reinterpret_cast<uint32_t *>(scratch + pt.fb_ranks);
       int *unit_max = reinterpret_cast<int *>(scratch + pt.unit_max);
       g.d_queries = reinterpret_cast<QueryDesc *>(base + pt.desc);
@@ -1097,7 +1125,8 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       g.d_mix = reinterpret_cast<uint32_t *>(base + pt.mix);
       if (g.mix) memcpy(&host[pt.mix], g.mix_lanes.data(), 4 * g.mix_lanes.size());
       if (!pt.units.empty()) memcpy(&host[pt.unit_tables], pt.units.data(), 4 * pt.units.size());
-      std::vector<QueryDesc> fq;
+      const uint32_t few = g.next && g.next->next ? (uint32_t)(ctx->num_sms * kRescoreWidePerSm) : 0u;
+      std::vector<QueryDesc> fq, wq;   // of the last rescoring launch, of the one on 32 lanes
       for (size_t i = 0; i < nq; ++i) {
         QueryDesc &q = kv.second[i];
         q.unit_done = unit_done + i * g.n_long;
@@ -1108,21 +1137,30 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
         if (!q.table) continue;
         QueryDesc f = q;
         if (g.next->mode == MODE_LONG_MSV) {
-          f.table = fb_table[kv.first][i].ptr;
+          f.table = fb_table[kv.first][i].t.ptr;
           f.seg_words = fb_seg_words[kv.first][i];
         } else {
-          set_table(f, fb_table[kv.first][i]);
+          set_table(f, fb_table[kv.first][i].t);
         }
         f.ranks = q.fallback_ranks;
         f.n_ranks = q.fallback_count;
+        f.more_than = few;
         fq.push_back(f);
+        if (!few) continue;
+        set_table(f, pt.wide[i]);
+        f.more_than = 0;
+        f.at_most = few;
+        wq.push_back(f);
       }
       memcpy(&host[pt.desc], kv.second.data(), sizeof(QueryDesc) * nq);
-      if (g.next) {
-        memcpy(&host[pt.fb_desc], fq.data(), sizeof(QueryDesc) * fq.size());
-        g.next->d_queries = reinterpret_cast<QueryDesc *>(base + pt.fb_desc);
-        g.next->d_counter = zero + 1;
-        g.next->d_units = g.d_units;
+      size_t at = pt.fb_desc, counter = 1;
+      for (LaunchGroup *x = g.next.get(); x; x = x->next.get()) {
+        const std::vector<QueryDesc> &d = x->next ? wq : fq;
+        memcpy(&host[at], d.data(), sizeof(QueryDesc) * d.size());
+        x->d_queries = reinterpret_cast<QueryDesc *>(base + at);
+        at += sizeof(QueryDesc) * d.size();
+        x->d_counter = zero + counter++;
+        x->d_units = g.d_units;
       }
     }
     e = cudaMemcpyAsync(pl->d_mem, host.data(), up.bytes, cudaMemcpyHostToDevice, ctx->stream);

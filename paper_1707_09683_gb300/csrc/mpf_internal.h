@@ -128,6 +128,7 @@ struct QueryDesc {
   // (a device count written by an earlier kernel on the same stream).
   const uint32_t *ranks;
   const uint32_t *n_ranks;
+  uint32_t more_than, at_most;   // of rank lists: score only more than, and (not 0) at most so many ranks
   // Tiled MSV kernel and MSV_HELD: sequences left to an exact kernel (their
   // length ranks, and the count, zero before the launch).
   uint32_t *fallback_ranks;

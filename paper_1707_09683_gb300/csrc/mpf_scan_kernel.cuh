@@ -292,7 +292,10 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
     }
     // A shard without sequences (a short rank list, such as the few
     // sequences a held MSV pass leaves for rescoring) stages nothing.
-    if ((uint64_t)shard >= (qd->ranks ? (uint64_t)*qd->n_ranks : (uint64_t)p.n_units)) {
+    // So does a query whose list another launch takes.
+    const uint64_t n_sel = qd->ranks ? (uint64_t)*qd->n_ranks : (uint64_t)p.n_units;
+    if ((uint64_t)shard >= n_sel ||
+        (qd->ranks && (n_sel <= qd->more_than || (qd->at_most && n_sel > qd->at_most)))) {
       __syncthreads();
       continue;
     }
@@ -371,7 +374,6 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         (MIX ? reinterpret_cast<const uint8_t *>(qd->table) : tbl_base) + qd->smax_off);
     auto gmax = [&](int x) { return MIX ? mixed_max(x, lane, gl, width) : group_max<LG>(x); };
     const uint32_t *ranks = qd->ranks;
-    const uint64_t n_sel = ranks ? (uint64_t)*qd->n_ranks : (uint64_t)p.n_units;
 
     for (;;) {
       // ---- take G consecutive length ranks of this shard (one per group;
