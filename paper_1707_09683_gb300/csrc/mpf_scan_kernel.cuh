@@ -242,6 +242,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   // Every lane of a warp follows the same sequence: a warp reduction (whose
   // result is uniform) hands each residue word to the rows.
   constexpr bool kUniform = TM != TM_NONE;
+  constexpr bool kTwoWords = kUniform && !kFast;
   // Mixed sets: item i scores set i / n_shards, whose lanes belong to queries
   // as p.mix_lanes says (query, lane of its group, width; width 0: no query).
   const uint32_t n_items = (MIX ? p.n_sets : (p.n_queries + QP - 1) / QP) * p.n_shards;
@@ -638,6 +639,31 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       if constexpr (TM) tm_ld_pow2<HI>(thi, tm_col(cur & 0xffu) + LO);   // first row
 
       int since_clear = 0;
+      if constexpr (kTwoWords) {
+        // Two words per turn, loaded a turn ahead (unguarded: at most three
+        // words past the rows, which lie in the database and are not scored).
+        const uint32_t *wp = p.residues + wptr;
+        uint32_t a1 = ahead, a2 = __ldg(wp + 2);
+        for (int step = 0; step < wsteps; step += 2) {
+          const uint32_t n1 = __reduce_max_sync(kFull, a1), n2 = __reduce_max_sync(kFull, a2);
+          a1 = __ldg(wp + step + 3);
+          a2 = __ldg(wp + step + 4);
+          four_rows(step, std::false_type{}, n1);
+          cur = n1;
+          if (step + 1 < wsteps) {
+            four_rows(step + 1, std::false_type{}, n2);
+            cur = n2;
+          }
+          if constexpr (kPair) {
+            since_clear += 2;
+            if (since_clear == kClearSteps) {
+              since_clear = 0;
+#pragma unroll
+              for (int q = 0; q < H; ++q) v[q] &= kCellMask2;
+            }
+          }
+        }
+      } else
       for (int step = 0; step < wsteps; ++step) {
         // Prefetch the residue words; past the end a group reads padding.
         const uint32_t nxt = kUniform ? __reduce_max_sync(kFull, ahead) : ahead;
