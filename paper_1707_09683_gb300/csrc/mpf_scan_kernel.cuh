@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   // result is uniform) hands each residue word to the rows.
   constexpr bool kUniform = TM != TM_NONE;
   constexpr bool kTwoWords = kUniform && !kFast;
+  constexpr bool kMapPad = TM == TM_FEW && HT == H;
   // Mixed sets: item i scores set i / n_shards, whose lanes belong to queries
   // as p.mix_lanes says (query, lane of its group, width; width 0: no query).
   const uint32_t n_items = (MIX ? p.n_sets : (p.n_queries + QP - 1) / QP) * p.n_shards;
@@ -453,7 +454,13 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       uint32_t tlo[LOW], thi[HI > 0 ? HI : 1];
       auto tm_col = [&](uint32_t xc) -> uint32_t {
         if (!MPF_DCHECK(p.status, xc < (uint32_t)kTableRows)) xc = kPadCode;
-        return tm_lane + (TM == TM_FEW ? min(xc, tm_pad) : xc) * (uint32_t)HT;
+        return tm_lane + (TM == TM_FEW && !kMapPad ? min(xc, tm_pad) : xc) * (uint32_t)HT;
+      };
+      uint32_t tcol = 0;       // TMEM column of the current row's words
+      // Lanes held whole in TMEM: padding codes become their TMEM row a word
+      // at a time (bit 5 marks them: the database's codes are below 20).
+      auto map_pad = [&](uint32_t w) {
+        return kMapPad ? w - ((w >> 5) & 0x01010101u) * ((uint32_t)kPadCode - tm_pad) : w;
       };
       // Four rows of one residue word (nxt: the next word).  CHECK: test every
       // row for the MSV threshold (only needed when some lane is near it, or
@@ -470,7 +477,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
           if (!MPF_DCHECK(p.status, x < (uint32_t)kTableRows)) x = kPadCode;
           if constexpr (TM) {
             tm_wait_ld<HI>(thi);
-            tm_ld_pow2<LOW>(tlo, tm_col(x));
+            tm_ld_pow2<LOW>(tlo, tcol);
           }
           const uint8_t *rowp = tbl_lane + x * row_bytes;
           // Diagonal shift (Alg. 5): cell k-1 of the previous row feeds cell k.
@@ -545,7 +552,8 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
               fold(LO + q - 1);
             }
             tm_wait_ld<LOW>(tlo);
-            tm_ld_pow2<HI>(thi, tm_col(rr < 3 ? __byte_perm(cur, 0u, 0x4440u + rr + 1) : nxt & 0xffu) + LO);
+            tcol = tm_col(rr < 3 ? __byte_perm(cur, 0u, 0x4440u + rr + 1) : nxt & 0xffu);
+            tm_ld_at<HI, LO>(thi, tcol);
 #pragma unroll
             for (int q = LO - 1; q >= 1; q -= 2) {
               cell(q, tlo[q]);
@@ -636,7 +644,11 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       cur = __ldg(p.residues + (nsteps > 0 ? wptr : p.pad_word));
       if constexpr (kUniform) cur = __reduce_max_sync(kFull, cur);
       ahead = __ldg(p.residues + (1 < nsteps ? wptr + 1u : p.pad_word));
-      if constexpr (TM) tm_ld_pow2<HI>(thi, tm_col(cur & 0xffu) + LO);   // first row
+      if constexpr (TM) {   // first row
+        cur = map_pad(cur);
+        tcol = tm_col(cur & 0xffu);
+        tm_ld_at<HI, LO>(thi, tcol);
+      }
 
       int since_clear = 0;
       if constexpr (kTwoWords) {
@@ -645,7 +657,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
         const uint32_t *wp = p.residues + wptr;
         uint32_t a1 = ahead, a2 = __ldg(wp + 2);
         for (int step = 0; step < wsteps; step += 2) {
-          const uint32_t n1 = __reduce_max_sync(kFull, a1), n2 = __reduce_max_sync(kFull, a2);
+          const uint32_t n1 = map_pad(__reduce_max_sync(kFull, a1)), n2 = map_pad(__reduce_max_sync(kFull, a2));
           a1 = __ldg(wp + step + 3);
           a2 = __ldg(wp + step + 4);
           four_rows(step, std::false_type{}, n1);

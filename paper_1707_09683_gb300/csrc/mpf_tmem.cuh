@@ -84,6 +84,21 @@ __device__ __forceinline__ void tm_ld_pow2<1>(uint32_t *r, uint32_t a) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[0]) : "r"(a));
 }
 
+// Eight or four columns starting OFF past column address a (as an immediate,
+// so that loads at one address share its uniform register).
+template <int N, int OFF>
+__device__ __forceinline__ void tm_ld_at(uint32_t *r, uint32_t a) {
+  static_assert(N == 8 || N == 4, "columns per load");
+  if constexpr (N == 8)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8 + %9];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(a), "n"(OFF));
+  else
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4 + %5];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a), "n"(OFF));
+}
+
 // N (< 32) consecutive columns starting at column address a.
 template <int N>
 __device__ __forceinline__ void tm_ld(uint32_t *r, uint32_t a) {
