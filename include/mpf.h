@@ -271,8 +271,8 @@ int mpf_scan_batch(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, in
  * Packed queries are sorted by words per lane; runs of them form sets where
  * a cost model in warp-words per row says a set pays, and each takes the
  * largest word count of its set (the added nodes score as padding: the
- * outputs do not change).  Queries left over whose configuration was never
- * set may share warps in mixed sets, each with as many lanes as its nodes
+ * outputs do not change).  Queries left over whose configuration is the
+ * default one may share warps in mixed sets, each with as many lanes as its nodes
  * need at the set's words per lane (databases whose codes are all below 20).
  *   mpf_plan_create:  arguments as mpf_scan_batch; raw/overflow/nat must be
  *                     device pointers (MPF_EINVAL otherwise).  The plan keeps

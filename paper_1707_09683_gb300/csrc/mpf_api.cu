@@ -733,7 +733,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     const mpf_profile *p;
     QueryDesc q;
     DevTable fb;
-    bool by_default;   // no configuration was set: it may join a mixed set
+    bool by_default;   // the configuration is the default one: it may join a mixed set
   };
   std::map<int, std::vector<QpCand>> mix_cand;   // by mode
   std::map<GroupKey, std::vector<uint32_t>> mix_lanes;
@@ -864,7 +864,9 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     if (n_q >= 2 && !ranks && !p->seg_words && lanes < 32 &&
         (mode == MODE_SSV || mode == MODE_MSV_HELD || mode == MODE_MSV_SSV) && words >= kTmMinWords &&
         p->table_mem[f] != MPF_TABLE_SHARED) {
-      qp_cand[std::make_pair(lanes, mode)].push_back(QpCand{words, sf, p, q, fb, p->cfg_lanes[f] == 0});
+      int dl = 0, dw = 0;
+      default_config(ctx, p->M, mode, &dl, &dw);
+      qp_cand[std::make_pair(lanes, mode)].push_back(QpCand{words, sf, p, q, fb, lanes == dl && words == dw});
       continue;
     }
     const GroupKey key(lanes, words, mode, tm, 1);

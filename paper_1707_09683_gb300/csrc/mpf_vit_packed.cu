@@ -161,6 +161,10 @@ __global__ void __launch_bounds__(block_threads(QH, TEAM), block_min(QH, TEAM))
     const VitPackTables &tb = TEAM ? Q.pk_team : Q.pk_solo;
     if (!MPF_DCHECK(p.status, n_sel <= p.n_seqs && tb.words == W * QH)) continue;
 
+    // Lanes of few words add every match score in two steps, which costs no
+    // more than the test and the branch on the residue's code.
+    constexpr bool kAlways = !TEAM && QH <= 2;
+
     // ---- this lane's transitions and the query's constants ----
     const uint32_t *tp = tb.trans + ((size_t)w * QH) * 32 + lane;
     const size_t plane = (size_t)W * QH * 32;
@@ -265,7 +269,7 @@ __global__ void __launch_bounds__(block_threads(QH, TEAM), block_min(QH, TEAM))
 
       // Short lanes load a row's match scores while the row before ends, long
       // ones a few words ahead.
-      uint32_t M[QH], I[QH], e[TM ? 1 : QH];
+      uint32_t M[QH], I[QH], e[TM ? 1 : QH], f[kAlways ? QH : 1];
 #pragma unroll
       for (int j = 0; j < QH; ++j) M[j] = I[j] = F2;
       uint32_t pM = F2, pI = F2, pD = F2;   // previous row: M, I, true D of the node before each half
@@ -275,17 +279,22 @@ __global__ void __launch_bounds__(block_threads(QH, TEAM), block_min(QH, TEAM))
       uint32_t xbm = pack16(max(lo, kFloor), max(lo, kFloor));
       int result = 0;     // 1 overflow, 2 left to the 32-bit kernel
       // Residues: the current word, shifted as its rows are used, and the
-      // next one.  Match scores are loaded a row ahead; the load after the
-      // last row takes whatever code follows (at most the padding code, whose
-      // row lies inside the table's second half) and is not used.
+      // next one (loads reach two words past the sequence, inside the
+      // database's spare words).  Match scores are loaded a row ahead; the load after the
+      // last row takes whatever code follows (at most the padding code 32,
+      // whose row is the second half's first, or row 31 where both halves are
+      // read) and is not used.
       const uint32_t *res = p.residues + w0;
-      uint32_t word = __ldg(res), wnext = __ldg(res + (len > 4 ? 1 : 0));
+      uint32_t word = __ldg(res), wnext = __ldg(res + 1);
       uint32_t x = word & 0xffu;
       auto load_scores = [&]() {
-        const uint32_t *er = emis + x * erow;
+        const uint32_t *er = emis + (kAlways ? min(x, kVitRows - 1u) : x) * erow;
         if constexpr (!TM) {
 #pragma unroll
-          for (int j = 0; j < QH; ++j) e[j] = __ldg(er + j * 32);
+          for (int j = 0; j < QH; ++j) {
+            e[j] = __ldg(er + j * 32);
+            if constexpr (kAlways) f[j] = __ldg(er + kVitRows * erow + j * 32);
+          }
         }
       };
       load_scores();
@@ -321,7 +330,10 @@ __global__ void __launch_bounds__(block_threads(QH, TEAM), block_min(QH, TEAM))
             best = addmax2(dI, t[kIM], best);
             best = addmax2(dD, t[kDM], best);
             uint32_t Mn = addmax2(best, ej, F2);
-            if constexpr (decltype(split_tag)::value) Mn = addmax2(Mn, ld_ordered(e2 + j * 32), F2);
+            if constexpr (kAlways)
+              Mn = addmax2(Mn, f[j], F2);
+            else if constexpr (decltype(split_tag)::value)
+              Mn = addmax2(Mn, ld_ordered(e2 + j * 32), F2);
             const uint32_t In = addmax2(I[j], t[kII], addmax2(M[j], t[kMI], F2));
             if (j > 0) d = addmax2(d, t[kDD], addmax2(mprev, t[kMD], F2));
             if (j & 1)
@@ -336,18 +348,17 @@ __global__ void __launch_bounds__(block_threads(QH, TEAM), block_min(QH, TEAM))
             mprev = Mn;
           }
         };
-        if ((split >> x) & 1u)
+        if constexpr (kAlways)
+          sweep(std::true_type{});
+        else if ((split >> x) & 1u)
           sweep(std::true_type{});
         else
           sweep(std::false_type{});
 
         // The next row's residue and match scores.
-        if ((i & 3) == 3) {
-          word = wnext;
-          if (i + 5 < len) wnext = __ldg(res + ((i >> 2) + 2));
-        } else {
-          word >>= 8;
-        }
+        const bool turn = (i & 3) == 3;
+        word = turn ? wnext : word >> 8;
+        if (turn) wnext = __ldg(res + ((i >> 2) + 2));
         x = word & 0xffu;
         if (!MPF_DCHECK(p.status, x <= (uint32_t)kVitRows)) x = 0;
         load_scores();

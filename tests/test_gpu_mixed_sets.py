@@ -1,6 +1,6 @@
 """Plans whose shorter queries share warps in mixed sets (bit-exact against the oracle).
 
-Queries without a set configuration and fewer than 32 lanes each get as many
+Queries of the default configuration and fewer than 32 lanes each get as many
 lanes of a warp as their nodes need: sets that fill the warp and sets that do
 not, groups of one lane, ragged last lanes, strong profiles (overflow, J
 chaining and its rescoring launch), per-code best scores for sequences whose
