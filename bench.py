@@ -154,24 +154,28 @@ SMEM_B_PER_CLK = 128.0
 TMEM_B_PER_CLK = 385.7
 ALU_LANES_PER_CLK = 64.0
 FMA_LANES_PER_CLK = 64.0
-TM_WORDS_ALL, TM_WORDS_PART = 14, 12   # words per lane from TMEM (all up to 14, else 12)
+TM_WORDS = 24   # words per lane from TMEM at most (databases of few codes, as the synthetic ones)
+TM_WORDS_F16 = (14, 12)   # fp16 cells: all up to 14, else 12
 
 
 def design_ceiling(filt, lanes, words, tm, f16, m, nsm, sm_mhz):
     """Ceiling of a striped kernel configuration in GCUPS (model cells): the
     lowest of its table-read and cell-update limits per SM clock, times the
     model's share of the padded cells.  Per 32-bit word (two cells) and DP
-    row: 4 B of table (from TMEM for the first 12 or 14 words of a lane
-    with tm, else from shared memory), one cell update (DPX on the ALU pipe, or
-    HFMA2 on the FMA pipe) and half a 3-input max (ALU)."""
-    ht = (words if words <= TM_WORDS_ALL else TM_WORDS_PART) if tm else 0
+    row: 4 B of table (with tm from TMEM for a lane's first words, else from
+    shared memory), half a cell update on the ALU pipe (DPX, every second row)
+    and half on the FMA pipe (integer multiply-add), or one HFMA2 on the FMA
+    pipe with fp16 cells, and half a 3-input max (ALU)."""
+    ht = min(words, TM_WORDS) if tm else 0
+    if tm and f16:
+        ht = words if words <= TM_WORDS_F16[0] else TM_WORDS_F16[1]
     lim = {}
     smem_b = 4.0 * (words - ht) / words
     if smem_b > 0:
         lim["shared-memory table reads"] = SMEM_B_PER_CLK / smem_b * 2
     if ht:
         lim["TMEM table reads"] = TMEM_B_PER_CLK / (4.0 * ht / words) * 2
-    alu_ops = 0.5 + (0.0 if f16 else 1.0)
+    alu_ops = 0.5 + (0.0 if f16 else 0.5)
     lim["ALU pipe (cell update + running max)" if not f16 else "ALU pipe (running max)"] = \
         ALU_LANES_PER_CLK / alu_ops * 2
     if f16:
@@ -605,7 +609,7 @@ def run_mpf(args):
                        "form": "batched persistent plan per filter, CUDA-graph replay",
                        "cell_arith": ("fp16 cells holding exact integers, HFMA2.RELU on the FMA pipe"
                                       if args.arith == "f16" else
-                                      "16-bit integer cells, two per register, DPX on the integer pipe; "
+                                      "16-bit integer cells, two per register, DPX and integer multiply-adds; "
                                       "exact byte semantics of Alg. 2 / Alg. 7; no floating point"),
                        "table_memory": args.table,
                        "kernel_configs": tuned or "default",
@@ -642,10 +646,11 @@ def run_mpf(args):
         dist.destroy_process_group()
 
 
-# DPX operations per cell of the saturating Viterbi recurrence once every
-# sat() is a single add-then-max (moves <= 0): 4 for the best predecessor of
-# M, 1 for the emission, 2 for I, 2 for D, 1 for the E maximum.
-VIT_OPS_PER_CELL = 10
+# DPX lane-operations per cell of the packed Viterbi kernel, two cells per
+# 16x2 lane: 3 for the predecessors of M beside the entry score, 1 for the
+# match score, 2 for I, 4 for the delete chains (the previous row's completed,
+# and this row's), half for the row maximum.
+VIT_OPS_PER_CELL = 10.5 / 2
 
 
 def run_viterbi_stage(args, ctx, db, wl, profs, p_msv, thr, run_pipe, time_steps, clocks, dev):
@@ -680,7 +685,7 @@ def run_viterbi_stage(args, ctx, db, wl, profs, p_msv, thr, run_pipe, time_steps
             "ms_per_step": ms_vit, "msv_min_nat": thr, "pairs_scored": passed,
             "pass_fraction": passed / (q * n), "cells_per_step": cells,
             "three_stage_ms_per_step": ms_three,
-            "kernel": "viterbi_fast_kernel (all moves <= 0)",
+            "kernel": "viterbi_packed_kernel (all moves <= 0, uniform entry; two nodes per register)",
             "roofline": {"bound": "alu", "achieved": gcups, "peak": peak, "unit": "GCUPS",
                          "frac": gcups / peak, "traffic": None,
                          "timed": "mpf_viterbi_rescore per step (3 selection kernels + 1 Viterbi kernel)",
@@ -718,8 +723,8 @@ def run_long_model(args, ctx, db, wl, time_steps, clocks, dev):
         log(f"long model M={args.long_m}: {name} {g:.1f} GCUPS ({ms:.1f} ms per launch)")
     prof.close()
     out["roofline_basis"] = "integer-SIMD roofline of the striped kernels (same formula as roofline.peak)"
-    # P7Viterbi on the same model length (DP rows in device memory), one
-    # query against the first sequences of the database.
+    # P7Viterbi on the same model length, one query against the first
+    # sequences of the database.
     k = min(args.long_vit_seqs, wl.db.n_seqs)
     vdb = mpf.Database(ctx, wl.db.residues, wl.db.offsets[:k], wl.db.lengths[:k])
     vp = mpf.VitProfile(ctx, synth.make_vit_profile(args.long_m, np.random.default_rng(901)))
@@ -733,7 +738,7 @@ def run_long_model(args, ctx, db, wl, time_steps, clocks, dev):
     peak = nsm * INT_LANES_PER_SM_CLK / VIT_OPS_PER_CELL * sm_mhz * 1e6 / 1e9
     out["viterbi"] = {"gcups": g, "ms_per_launch": ms, "n_seqs": k, "cells_per_launch": cells,
                       "roofline_frac": g / peak, "peak": peak,
-                      "kernel": "viterbi_fast_kernel, DP rows in device memory"}
+                      "kernel": "viterbi_packed_kernel (teams of warps)"}
     log(f"long model M={args.long_m}: viterbi {g:.1f} GCUPS on {k} sequences ({ms:.1f} ms per launch)")
     vp.close()
     vdb.close()

@@ -140,8 +140,9 @@ void mpf_profile_destroy(mpf_profile *prof);
  * sequences per warp, W = 2 * lanes cells per row step, H = words).
  * set: MPF_EINVAL if the pair is not built or does not cover M, or if the
  *      profile is longer than mpf_max_striped_length() (one configuration).
- * get: writes the pair the next scan will use (tuned default if never set);
- *      lanes 32, words 0 for the long-model kernel.
+ * get: writes the pair the next scan will use (tuned default if never set,
+ *      where a scan may take a whole-warp kernel or a plan a mixed set instead:
+ *      mpf_plan_group_info); lanes 32, words 0 for the long-model kernel.
  */
 int mpf_profile_set_config(mpf_profile *prof, int filter, int lanes, int words);
 int mpf_profile_get_config(const mpf_profile *prof, int filter, int *lanes, int *words);

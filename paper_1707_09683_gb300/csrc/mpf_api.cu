@@ -93,6 +93,19 @@ void default_config(const mpf_ctx *ctx, int M, int mode, int *lanes, int *words)
   *words = 0;
 }
 
+// Words per lane of the whole-warp kernel that scores a query of a narrower
+// default configuration when it is alone in a warp, or 0.  Above kAloneTmM
+// nodes the tensor-memory kernel is ahead of the narrow groups, whose rows
+// are bound by shared-memory reads (SSV, 60,000 sequences, ms narrow / whole
+// warp: M = 448 0.56 / 0.54, 512 0.64 / 0.54, 640 0.81 / 0.65, 800 0.98 / 0.79,
+// 1,024 1.28 / 0.91).
+constexpr int kAloneTmM = 448;
+int alone_words(int M, int mode) {
+  if (M <= kAloneTmM || (mode != MODE_SSV && mode != MODE_MSV_HELD && mode != MODE_MSV_SSV)) return 0;
+  const int w = (M + 127) / 128 * 2;
+  return w >= kTmMinWords && w <= kMaxWords && kernel_lg32_tm(w, mode) ? w : 0;
+}
+
 // MSV_FAST needs the first begin score of every sequence below 255 - bias.
 bool msv_fast_ok(const mpf_profile *p) {
   int xb = p->base - (p->tjb_min + p->tbm);
@@ -380,12 +393,16 @@ bool use_tmem(const mpf_profile *p, int filter, int lanes, int words, int mode) 
 // queries alone is dissolved.
 struct MixQuery {
   int M, lanes, words;   // with its default configuration
+  int whole;             // words of the whole-warp kernel it takes when left alone, or 0
 };
 std::pair<int, std::vector<std::vector<int>>> mix_sets(const std::vector<MixQuery> &qs) {
   std::vector<int> order(qs.size());
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return qs[a].M > qs[b].M; });
-  auto alone = [&](int i) { return 1.25 * qs[i].words * qs[i].lanes / 32.0 + 3.0; };
+  auto alone = [&](int i) {
+    const double narrow = 1.25 * qs[i].words * qs[i].lanes / 32.0 + 3.0;
+    return qs[i].whole ? std::min(narrow, qs[i].whole + 2.7) : narrow;
+  };
   std::pair<int, std::vector<std::vector<int>>> best(0, {});
   double saved_best = 0;
   for (int H = kMixWordsMin; H <= kMixWordsMax; H += 2) {
@@ -733,6 +750,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     const mpf_profile *p;
     QueryDesc q;
     DevTable fb;
+    bool unset;        // no configuration was set
     bool by_default;   // the configuration is the default one: it may join a mixed set
   };
   std::map<int, std::vector<QpCand>> mix_cand;   // by mode
@@ -812,7 +830,16 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     } else {
       lanes = p->cfg_lanes[f];
       words = p->cfg_words[f];
-      if (!lanes) default_config(ctx, p->M, mode, &lanes, &words);
+      if (!lanes) {
+        default_config(ctx, p->M, mode, &lanes, &words);
+        // With others to share a warp with, that is decided below.
+        const int w = lanes < 32 && (n_q == 1 || ranks) && p->table_mem[f] != MPF_TABLE_SHARED
+                          ? alone_words(p->M, mode) : 0;
+        if (w) {
+          lanes = 32;
+          words = w;
+        }
+      }
       if (!lanes || !kernel_for(lanes, words, mode)) {
         plan_free(pl);
         return MPF_EUNSUPPORTED;
@@ -866,7 +893,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
         p->table_mem[f] != MPF_TABLE_SHARED) {
       int dl = 0, dw = 0;
       default_config(ctx, p->M, mode, &dl, &dw);
-      qp_cand[std::make_pair(lanes, mode)].push_back(QpCand{words, sf, p, q, fb, lanes == dl && words == dw});
+      qp_cand[std::make_pair(lanes, mode)].push_back(QpCand{words, sf, p, q, fb, p->cfg_lanes[f] == 0, lanes == dl && words == dw});
       continue;
     }
     const GroupKey key(lanes, words, mode, tm, 1);
@@ -893,7 +920,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       const size_t a = r.first, b = r.second;
       const bool pack = b - a >= 2;
       const int H = v[b - 1].words;
-      if (!pack && v[a].by_default && db->code_end <= kTmFewCodes) {
+      if (!pack && v[a].by_default) {
         mix_cand[mode].push_back(v[a]);
         continue;
       }
@@ -926,7 +953,8 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       }
     }
   }
-  // Mixed sets of the queries that are left over.  Their rescoring launch
+  // Mixed sets of the queries that are left over, and what those still alone
+  // take.  Their rescoring launch
   // (one query per warp) takes 32 lanes, with the words that the longest needs.
   for (auto &kv : mix_cand) {
     const int mode = kv.first;
@@ -935,9 +963,10 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     for (const QpCand &c : v) {
       int lanes = 0, words = 0;
       default_config(ctx, c.p->M, mode, &lanes, &words);
-      mq.push_back(MixQuery{c.p->M, lanes, words});
+      mq.push_back(MixQuery{c.p->M, lanes, words, c.unset ? alone_words(c.p->M, mode) : 0});
     }
-    const auto mix = mix_sets(mq);
+    auto mix = std::make_pair(0, std::vector<std::vector<int>>());
+    if (db->code_end <= kTmFewCodes) mix = mix_sets(mq);
     std::vector<bool> placed(v.size(), false);
     int longest = 1;
     for (const auto &set : mix.second)
@@ -970,7 +999,18 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     }
     for (size_t i = 0; i < v.size(); ++i) {
       if (placed[i]) continue;
-      const GroupKey alone(mq[i].lanes, mq[i].words, mode, 0, 1);
+      const int w = mq[i].whole;
+      if (w) {
+        DevTable t;
+        const int rc = get_table(v[i].p, 32, w, TABLE_I16, &t);
+        if (rc) {
+          plan_free(pl);
+          return rc;
+        }
+        set_table(v[i].q, t);
+        v[i].fb = t;
+      }
+      const GroupKey alone(w ? 32 : mq[i].lanes, w ? w : mq[i].words, mode, w ? 1 : 0, 1);
       byconf[alone].push_back(v[i].q);
       if (mode != MODE_SSV) fb_table[alone].push_back(Rescore{v[i].fb, v[i].p});
       group_shards[alone] = std::max(group_shards[alone], v[i].sf);
