@@ -40,14 +40,23 @@ def test_long_weak_diagonals_across_tiles(M):
     check(M, 20, np.random.default_rng(M))
 
 
-def check(M, codes, rng, lanes=0, words=0):
+@pytest.mark.parametrize("M", [3073, 4100])
+def test_tile_rows_left_over_after_turns_of_eight(M):
+    """Every remainder of a tile's turns of eight rows, before and around a clearing row."""
+    check(M, 20, np.random.default_rng(8 * M), lengths=[*range(20), *range(112, 130)])
+
+
+LENGTHS = [3, 119, 120, 121, 122, 240, 243, 1201, 0, 1, 777, 2, 1802]
+
+
+def check(M, codes, rng, lanes=0, words=0, lengths=LENGTHS):
     import torch
 
     import oracle
     from paper_1707_09683_gb300 import mpf
 
     p = weak_profile(M, rng, codes)
-    lengths = np.array([3, 119, 120, 121, 122, 240, 243, 1201, 0, 1, 777, 2, 1802], dtype=np.uint32)
+    lengths = np.array(lengths, dtype=np.uint32)
     offsets = np.concatenate([[0], np.cumsum(lengths[:-1])]).astype(np.uint64)
     res = rng.integers(0, codes, size=int(lengths.sum())).astype(np.uint8)
     res[0] = codes - 1
