@@ -610,8 +610,10 @@ int configure_kernel(mpf_ctx *ctx, LaunchGroup *g) {
     if (!best_w) return MPF_EUNSUPPORTED;
     g->threads = best_w * 32;
     g->smem = (uint32_t)(per_warp * (size_t)best_w);
+    // The limit is the kernel's, not the plan's: plans of other model lengths
+    // launch the same kernel with other sizes.
     MPF_CUDA(cudaFuncSetAttribute((const void *)g->fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)g->smem));
+                                  ctx->max_smem));
     // The driver takes the smallest supported carveout at or above the
     // preference: ask for just under the chosen one.
     MPF_CUDA(cudaFuncSetAttribute((const void *)g->fn, cudaFuncAttributePreferredSharedMemoryCarveout,
