@@ -285,40 +285,40 @@ int get_long_table(const mpf_profile *p, const uint8_t **out) {
 }
 
 // Device copy of a long profile's scores for the tiled kernel: per tile of
-// kTileNodes nodes, [code][chunk][lane] x 4 pairs of int16, lane l's pair
-// p = (node l * kTileC + p, the same + kTileC / 2) of the tile, chunk p / 4;
+// 64 * words nodes, [code][chunk][lane] x 4 pairs of int16, lane l's pair
+// p = (node l * 2 * words + p, the same + words) of the tile, chunk p / 4;
 // s = bias - cost (codes >= K cost 255), -32768 past M; then the 32 per-code
 // maxima of s over the model.  scaled (the tensor-memory kernel): scores in
 // units of 2^kCellShift, kNegInf past M.
-int get_tile_table(const mpf_profile *p, bool scaled, const uint4 **out) {
+int get_tile_table(const mpf_profile *p, bool scaled, int words, const uint4 **out) {
   std::lock_guard<std::mutex> lk(p->mu);
-  auto key = std::make_tuple(32, 0, scaled ? 4 : 3);
+  auto key = std::make_tuple(32, words == kTileC / 2 ? 0 : words, scaled ? 4 : 3);
   auto it = p->tables.find(key);
   if (it != p->tables.end()) {
     *out = it->second.ptr;
     return MPF_OK;
   }
-  const int M = p->M, nt = (M + kTileNodes - 1) / kTileNodes;
-  constexpr int kChunks = kTileC / 8;
-  std::vector<int16_t> img((size_t)nt * kTileTableBytes / 2 + 32);
+  const int M = p->M, nt = (int)tiles_of(M, words);
+  const size_t chunks = (size_t)words / 4, tiles_len = (size_t)nt * tile_bytes(words) / 2;
+  std::vector<int16_t> img(tiles_len + 32);
   for (int x = 0; x < 32; ++x) {
     int m = p->bias - 255;
     if (x < p->K)
       for (int k = 0; k < M; ++k) m = std::max(m, p->bias - (int)p->cost[(size_t)x * M + k]);
-    img[(size_t)nt * kTileTableBytes / 2 + x] = (int16_t)m;
+    img[tiles_len + x] = (int16_t)m;
   }
   for (int t = 0; t < nt; ++t)
     for (int x = 0; x < 32; ++x)
       for (int l = 0; l < 32; ++l)
-        for (int c = 0; c < kTileC; ++c) {
-          const int k = t * kTileNodes + l * kTileC + c;
+        for (int c = 0; c < 2 * words; ++c) {
+          const int k = (t * 32 + l) * 2 * words + c;
           int16_t s = (int16_t)(scaled ? kNegInf : -32768);
           if (k < M) {
             const int sv = p->bias - (x < p->K ? (int)p->cost[(size_t)x * M + k] : 255);
             s = (int16_t)(scaled ? sv * (1 << kCellShift) : sv);
           }
-          const int pr = c % (kTileC / 2), half = c / (kTileC / 2);
-          const size_t chunk = (((size_t)t * 32 + x) * kChunks + pr / 4) * 32 + l;
+          const int pr = c % words, half = c / words;
+          const size_t chunk = (((size_t)t * 32 + x) * chunks + pr / 4) * 32 + l;
           img[chunk * 8 + (pr % 4) * 2 + half] = s;
         }
   mpf_ctx *ctx = p->ctx;
@@ -480,6 +480,24 @@ std::vector<std::pair<size_t, size_t>> pack_runs(int lanes, int mode, const std:
 
 // One launch of the scan kernel over a set of queries sharing a kernel
 // configuration.  Device arrays lie in the plan's allocation.
+// Where the tiles of a long model go: 0 shared memory, 1 tensor memory,
+// kTmWideTiles tensor memory in tiles of kWideTileWords words per lane, which
+// hold the rows of codes below kWideTileCodes only.  A row of a wide tile
+// costs 1.12 times a row of a tile of 16 words and updates 1.25 times the
+// cells, so wide tiles are taken where they cover the model with no more
+// nodes (and their table is no larger than mpf_profile_footprint says).  SSV,
+// 20,000 sequences, ms 16 / 20 words: M = 3,100 1.37 / 1.15, 3,500 1.37 /
+// 1.15, 5,000 1.71 / 1.53 (both filters 2.27 / 2.15); 5,000 sequences, M =
+// 10,000 2.64 / 2.40.
+constexpr int kTmWideTiles = 2;
+int tile_memory(const mpf_profile *p, int filter, const mpf_db *db) {
+  if (p->table_mem[filter] == MPF_TABLE_SHARED) return 0;
+  return db->code_end <= kWideTileCodes &&
+                 tiles_of(p->M, kWideTileWords) * kWideTileWords <= tiles_of(p->M, kTileC / 2) * (kTileC / 2)
+             ? kTmWideTiles
+             : 1;
+}
+
 struct LaunchGroup {
   KernelFn fn = nullptr;
   int lanes = 0, words = 0, mode = 0;
@@ -499,6 +517,7 @@ struct LaunchGroup {
   uint32_t *d_zero = nullptr;       // words zeroed before each launch (null: a fallback launch, zeroed with its group)
   size_t zero_words = 0;
   bool tm = false;                  // striped kernel with the table in tensor memory
+  bool wide_tiles = false;          // tile kernel with wide tiles in tensor memory
   int shard_factor = 1;             // striped kernels: shards = factor x resident blocks
   uint32_t n_real = 0;              // queries of the group (n_queries less empty slots of packed sets)
   int qp = 1;                       // tensor-memory kernels: queries scored per warp and sequence
@@ -558,7 +577,7 @@ int configure_kernel(mpf_ctx *ctx, LaunchGroup *g) {
     // (tm) one block of kTileWarpsTm warps per SM with the tile in TMEM: it
     // asks for more than half the shared memory so that no second block of
     // the kernel shares the SM.
-    g->fn = tile_kernel_fn(g->mode, g->tm);
+    g->fn = tile_kernel_fn(g->mode, g->tm, g->wide_tiles);
     g->threads = (g->tm ? kTileWarpsTm : kTileWarps) * 32;
     g->smem = g->tm ? (uint32_t)ctx->max_smem / 2 + 1024 : (uint32_t)kTileTableBytes;
     MPF_CUDA(cudaFuncSetAttribute((const void *)g->fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -798,15 +817,16 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     int lanes = 32, words = 0;
     if (mode == MODE_TILE_SSV || mode == MODE_TILE_MSV || mode == MODE_TILE_MSV_SSV) {
       const uint4 *tt = nullptr;
-      const int ttm = p->table_mem[f] == MPF_TABLE_SHARED ? 0 : 1;   // tiles in TMEM
-      int rc = get_tile_table(p, ttm != 0, &tt);
+      const int ttm = tile_memory(p, f, db);
+      const int tw = ttm == kTmWideTiles ? kWideTileWords : kTileC / 2;
+      int rc = get_tile_table(p, ttm != 0, tw, &tt);
       if (rc) {
         plan_free(pl);
         return rc;
       }
       q.table = tt;
       q.M = (uint32_t)p->M;
-      q.smax_off = (uint32_t)(((size_t)(p->M + kTileNodes - 1) / kTileNodes) * kTileTableBytes);
+      q.smax_off = (uint32_t)(tiles_of(p->M, tw) * tile_bytes(tw));
       if (mode != MODE_TILE_SSV) {   // the lane-segment kernel's table, for the fallback
         const uint8_t *lt = nullptr;
         rc = get_long_table(p, &lt);
@@ -887,7 +907,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     q.ranks = ranks ? ranks + off : nullptr;
     q.n_ranks = ranks ? n_ranks + i : nullptr;
     const bool tiled = mode == MODE_TILE_SSV || mode == MODE_TILE_MSV || mode == MODE_TILE_MSV_SSV;
-    const int tm = tiled ? (p->table_mem[f] == MPF_TABLE_SHARED ? 0 : 1)
+    const int tm = tiled ? tile_memory(p, f, db)
                          : p->seg_words ? 0 : (use_tmem(p, f, lanes, words, mode) ? 1 : 0);
     const int sf = p->seg_words ? 1 : p->shard_factor[f];
     if (n_q >= 2 && !ranks && !p->seg_words && lanes < 32 &&
@@ -1051,6 +1071,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     g.words = std::get<1>(kv.first);
     g.mode = std::get<2>(kv.first);
     g.tm = std::get<3>(kv.first) != 0;
+    g.wide_tiles = std::get<3>(kv.first) == kTmWideTiles;
     g.mix = std::get<4>(kv.first) == kMixedKey;
     if (g.mix) {
       g.mix_lanes = mix_lanes[kv.first];

@@ -188,9 +188,17 @@ constexpr int kTileNodes = 32 * kTileC;
 constexpr int kTileWarps = 8;
 constexpr int kTileWarpsTm = 16;
 constexpr size_t kTileTableBytes = (size_t)32 * kTileNodes * 2;   // per tile
+// Words (pairs) per lane of a tile: kTileC / 2, or kWideTileWords for the
+// tensor-memory variant with wide tiles, whose 512 columns hold the rows of
+// codes below kWideTileCodes.
+constexpr int kWideTileWords = 20;
+constexpr int kWideTileCodes = (int)(kTmemColumns / kWideTileWords);
+__host__ __device__ constexpr size_t tiles_of(int M, int words) { return ((size_t)M + 64 * words - 1) / (64 * words); }
+constexpr size_t tile_bytes(int words) { return (size_t)32 * 32 * words * 4; }
 // The tiled kernel for a mode (MODE_TILE_*); tm: the tensor-memory variant
-// (blocks of kTileWarpsTm warps, one per SM, the tile's scores in TMEM).
-KernelFn tile_kernel_fn(int mode, bool tm);
+// (blocks of kTileWarpsTm warps, one per SM, the tile's scores in TMEM); wide:
+// its tiles of kWideTileWords words per lane.
+KernelFn tile_kernel_fn(int mode, bool tm, bool wide);
 
 // Stage-to-stage hand-off (mpf_pipeline.cu): SSV -> MSV (raw_bytes 1) and
 // MSV -> Viterbi (raw_bytes 2).

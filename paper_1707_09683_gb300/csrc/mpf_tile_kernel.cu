@@ -88,26 +88,29 @@ __device__ __forceinline__ void tile_row(uint32_t (&v)[kPairs], uint32_t in, con
 // cells and scores in units of 2^kCellShift).
 
 // Pair 0's diagonal: the node before the segment is in the high half of
-// in_word (the lane before's pair 15, or a boundary-column word).
-__device__ __forceinline__ uint32_t first_cell(uint32_t in_word, const uint32_t (&v)[kPairs]) {
-  return __byte_perm(in_word, v[kPairs - 1], 0x5432);
+// in_word (the lane before's last pair, or a boundary-column word).
+template <int P>
+__device__ __forceinline__ uint32_t first_cell(uint32_t in_word, const uint32_t (&v)[P]) {
+  return __byte_perm(in_word, v[P - 1], 0x5432);
 }
 // First row: sums, not clamped.
-__device__ __forceinline__ void pair_row_first(uint32_t (&v)[kPairs], uint32_t in_word,
-                                               const uint32_t (&sc)[kPairs], uint32_t &rmax, uint32_t one) {
+template <int P>
+__device__ __forceinline__ void pair_row_first(uint32_t (&v)[P], uint32_t in_word, const uint32_t (&sc)[P],
+                                               uint32_t &rmax, uint32_t one) {
   const uint32_t d0 = first_cell(in_word, v);
 #pragma unroll
-  for (int p = kPairs - 1; p >= 0; --p) {
+  for (int p = P - 1; p >= 0; --p) {
     v[p] = add_imad(p > 0 ? v[p - 1] : d0, sc[p], one);
     if ((p & 1) == 0) rmax = __vimax3_s16x2(rmax, v[p + 1], v[p]);
   }
 }
 // Second row: both rows' clamps.
-__device__ __forceinline__ void pair_row_second(uint32_t (&v)[kPairs], uint32_t in_word,
-                                                const uint32_t (&sc)[kPairs], uint32_t &rmax) {
+template <int P>
+__device__ __forceinline__ void pair_row_second(uint32_t (&v)[P], uint32_t in_word, const uint32_t (&sc)[P],
+                                                uint32_t &rmax) {
   const uint32_t d0 = first_cell(in_word, v);
 #pragma unroll
-  for (int p = kPairs - 1; p >= 0; --p) {
+  for (int p = P - 1; p >= 0; --p) {
     v[p] = __viaddmax_s16x2_relu(p > 0 ? v[p - 1] : d0, sc[p], sc[p]);
     if ((p & 1) == 0) rmax = __vimax3_s16x2(rmax, v[p + 1], v[p]);
   }
@@ -328,11 +331,12 @@ __global__ void __launch_bounds__(kTileWarps * 32) tile_kernel(ScanParams sp) {
 // The tensor-memory variant: blocks of kTileWarpsTm warps, one block per SM
 // (it allocates all of the SM's TMEM columns).  The tile's scores are not
 // staged in shared memory: every lane quarter of TMEM holds the whole tile,
-// code x's kPairs words of lane l at columns x * kPairs .. + kPairs - 1 of
-// the quarter's lane l (32 codes x 16 words = the 512 columns), and warp w
+// code x's P words of lane l at columns x * P .. + P - 1 of the quarter's
+// lane l (32 codes x 16 words = the 512 columns, or 25 x 20), and warp w
 // reads quarter w mod 4.  Warp w fills codes 8 (w / 4) .. + 7 of its quarter
 // from the tile in device memory.  One sequence per warp makes the residue
-// code of a row warp-uniform, so a row's 16 words are one tcgen05.ld, issued
+// code of a row warp-uniform, so a row's P words are one or two tcgen05.ld
+// at one column address, issued
 // a row ahead into the other of two register buffers.
 //
 // The sweep keeps the largest cell V only, which decides MSV as in the striped
@@ -345,18 +349,26 @@ __global__ void __launch_bounds__(kTileWarps * 32) tile_kernel(ScanParams sp) {
 // Measured before / after, 20,000 sequences (M = 5,000: SSV 1.79 / 1.71 ms,
 // both filters 2.46 / 2.27; M = 3,500: SSV 1.43 / 1.37) and 5,000 (M =
 // 10,000: SSV 2.99 / 2.64).
-template <bool MSV, bool BOTH>
+template <int P>
+__device__ __forceinline__ void tile_ld(uint32_t (&r)[P], uint32_t a) {
+  static_assert(P == 16 || P == 20, "words per lane");
+  tm_ld_pow2<16>(r, a);
+  if constexpr (P == 20) tm_ld_at<4, 16>(r + 16, a);
+}
+
+template <bool MSV, bool BOTH, int P>
 __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParams sp) {
   static_assert(MSV || !BOTH, "the both-filter sweep is the MSV sweep");
-  static_assert(32 * kPairs == (int)kTmemColumns && kTileWarpsTm % 4 == 0, "a tile fills a lane quarter");
+  constexpr int kCodes = P == kPairs ? 32 : kWideTileCodes;   // rows in TMEM
+  static_assert(kCodes * P <= (int)kTmemColumns && kTileWarpsTm == 16, "a tile fits a lane quarter");
   __shared__ uint32_t s_item, s_tmem;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int W = blockDim.x >> 5;
-  constexpr int kTileWords = 32 * kChunks * 32;   // uint4 per tile
+  constexpr int kRowWords = P / 4 * 32, kTileWords = 32 * kRowWords;   // uint4 per code and per tile
   const uint64_t cw = (uint64_t)blockIdx.x * W + warp;
-  // Boundary columns of 32-bit words: position i + 1 holds row i's pair 15
-  // of lane 31 (node 31 in the high half), read by the next tile's lane 0.
+  // Boundary columns of 32-bit words: position i + 1 holds row i's last
+  // pair of lane 31 (its last node in the high half), read by the next tile's lane 0.
   uint32_t *colbuf = reinterpret_cast<uint32_t *>(sp.tile_col + cw * 2 * (uint64_t)sp.tile_col_stride);
   const uint32_t col_elems = sp.tile_col_stride / 4;
   // Debug builds: the block shape and the block's columns within their
@@ -405,7 +417,7 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
     const int tj = qd.tjb ? (int)__ldg(qd.tjb + min(len, qd.n_tjb - 1u)) : qd.tjb_fixed;
     const int b = min(min(255, max(0, qd.base - (tj + qd.tbm))), 255 - qd.bias);
     const int T = min(qd.base + qd.tec - b, 255 - qd.bias - b - 1);
-    const int nt = (int)((qd.M + kTileNodes - 1) / kTileNodes);
+    const int nt = (int)tiles_of((int)qd.M, P);
     uint32_t rmax = 0, rmax2 = 0;   // running maxima over second and first rows of pairs
     for (int t = 0; t < nt; ++t) {
       // Every thread waited for its loads of the previous tile: order them
@@ -417,14 +429,13 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
         const uint4 *g = qd.table + (size_t)t * kTileWords + lane;
         const int x0 = 8 * (warp >> 2);
 #pragma unroll 2
-        for (int x = x0; x < x0 + 8; ++x) {
-          const uint4 c0 = __ldg(g + x * 128), c1 = __ldg(g + x * 128 + 32), c2 = __ldg(g + x * 128 + 64),
-                      c3 = __ldg(g + x * 128 + 96);
-          const uint32_t col = tm_lane + (uint32_t)(x * kPairs);
-          tm_st4(col, c0.x, c0.y, c0.z, c0.w);
-          tm_st4(col + 4, c1.x, c1.y, c1.z, c1.w);
-          tm_st4(col + 8, c2.x, c2.y, c2.z, c2.w);
-          tm_st4(col + 12, c3.x, c3.y, c3.z, c3.w);
+        for (int x = x0; x < min(x0 + 8, kCodes); ++x) {
+          uint4 c[P / 4];
+#pragma unroll
+          for (int i = 0; i < P / 4; ++i) c[i] = __ldg(g + x * kRowWords + 32 * i);
+          const uint32_t col = tm_lane + (uint32_t)(x * P);
+#pragma unroll
+          for (int i = 0; i < P / 4; ++i) tm_st4(col + 4 * i, c[i].x, c[i].y, c[i].z, c[i].w);
         }
         tm_wait_st();
       }
@@ -436,9 +447,9 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
       uint32_t *cout = colbuf + (size_t)(t & 1) * col_elems;
       const bool first = t == 0, write = t + 1 < nt;
       if (write && lane == 31) cout[0] = 0;
-      uint32_t v[kPairs];
+      uint32_t v[P];
 #pragma unroll
-      for (int p = 0; p < kPairs; ++p) v[p] = 0u;
+      for (int p = 0; p < P; ++p) v[p] = 0u;
       // Residue words and boundary words (0 but in lane 0) of the rows ahead:
       // A, the next four rows, and B, the four after.  Each is loaded again as
       // soon as its rows are done, so a turn of eight rows moves no registers.
@@ -452,27 +463,27 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
         cB = __ldcg(reinterpret_cast<const uint4 *>(cin) + 1);
       }
       uint32_t wA = word_at(0), wB = word_at(4);
-      // Score rows of the current and the next row.  Codes are < 32 in a
-      // sequence; the load issued for the row after the last one takes any
+      // Score rows of the current and the next row.  Codes are < kCodes
+      // in a sequence; the load issued for the row after the last one takes any
       // code (only waited for).
-      uint32_t TA[kPairs], TB[kPairs];
-      tm_ld<kPairs>(TA, tm_lane + (wA & 255u) * (uint32_t)kPairs);
+      uint32_t TA[P], TB[P];
+      tile_ld<P>(TA, tm_lane + (wA & 255u) * (uint32_t)P);
       // One row: wait for its scores, issue the next row's load (code xn),
-      // update.  The lane before's node 31 (high half) of the previous row
+      // update.  The lane before's last node (high half) of the previous row
       // comes by shuffle; lane 0 takes the boundary word, by a multiply-add
       // on the FMA pipe.
-      auto one_row = [&](const int u, uint32_t (&Tc)[kPairs], uint32_t (&Tn)[kPairs], uint32_t xn, uint32_t c,
+      auto one_row = [&](const int u, uint32_t (&Tc)[P], uint32_t (&Tn)[P], uint32_t xn, uint32_t c,
                          uint32_t *out, bool last) {
-        tm_wait_ld<kPairs>(Tc);
-        tm_ld<kPairs>(Tn, tm_lane + xn * (uint32_t)kPairs);
-        const uint32_t in = __shfl_up_sync(kAll, v[kPairs - 1], 1) * not_first + c;
+        tm_wait_ld<P>(Tc);
+        tile_ld<P>(Tn, tm_lane + xn * (uint32_t)P);
+        const uint32_t in = __shfl_up_sync(kAll, v[P - 1], 1) * not_first + c;
         if (u & 1)
           pair_row_second(v, in, Tc, rmax);
         else
           pair_row_first(v, in, Tc, rmax2, sp.one);
         // The word handed on at the end of a turn carries no fraction past a
         // clearing row of the next tile.
-        if (bound_out) out[u + 1] = last ? v[kPairs - 1] & kCellMask2 : v[kPairs - 1];
+        if (bound_out) out[u + 1] = last ? v[P - 1] & kCellMask2 : v[P - 1];
       };
       auto four_rows = [&](uint32_t w, const uint4 &c, uint32_t wn, uint32_t *out, bool turn_end) {
         one_row(0, TA, TB, __byte_perm(w, 0u, 0x4441), c.x, out, false);
@@ -494,7 +505,7 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
         if (until_clear == 0) {   // drop the sums' carries
           until_clear = 4 * kClearSteps;
 #pragma unroll
-          for (int p = 0; p < kPairs; ++p) v[p] &= kCellMask2;
+          for (int p = 0; p < P; ++p) v[p] &= kCellMask2;
         }
       }
       if (i0 + 4 <= len) {
@@ -506,8 +517,8 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
       if (i0 < len) one_row(0, TA, TB, __byte_perm(wA, 0u, 0x4441), cA.x, cout + i0, false);
       if (i0 + 1 < len) one_row(1, TB, TA, __byte_perm(wA, 0u, 0x4442), cA.y, cout + i0, false);
       if (i0 + 2 < len) one_row(2, TA, TB, __byte_perm(wA, 0u, 0x4443), cA.z, cout + i0, false);
-      tm_wait_ld<kPairs>(TB);
-      tm_wait_ld<kPairs>(TA);   // the load issued after the last row
+      tm_wait_ld<P>(TB);
+      tm_wait_ld<P>(TA);   // the load issued after the last row
     }
     const int V = half_max(__vmaxs2(rmax, rmax2)) >> kCellShift;
     if (MSV) {
@@ -541,11 +552,15 @@ __global__ void __launch_bounds__(kTileWarpsTm * 32, 1) tile_kernel_tm(ScanParam
 
 }  // namespace
 
-KernelFn tile_kernel_fn(int mode, bool tm) {
+KernelFn tile_kernel_fn(int mode, bool tm, bool wide) {
+  if (tm && wide)
+    return mode == MODE_TILE_MSV_SSV ? tile_kernel_tm<true, true, kWideTileWords>
+           : mode == MODE_TILE_MSV   ? tile_kernel_tm<true, false, kWideTileWords>
+                                     : tile_kernel_tm<false, false, kWideTileWords>;
   if (tm)
-    return mode == MODE_TILE_MSV_SSV ? tile_kernel_tm<true, true>
-           : mode == MODE_TILE_MSV   ? tile_kernel_tm<true, false>
-                                     : tile_kernel_tm<false, false>;
+    return mode == MODE_TILE_MSV_SSV ? tile_kernel_tm<true, true, kPairs>
+           : mode == MODE_TILE_MSV   ? tile_kernel_tm<true, false, kPairs>
+                                     : tile_kernel_tm<false, false, kPairs>;
   return mode == MODE_TILE_MSV_SSV ? tile_kernel<true, true> : mode == MODE_TILE_MSV ? tile_kernel<true> : tile_kernel<false>;
 }
 

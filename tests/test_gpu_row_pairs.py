@@ -40,10 +40,12 @@ def test_long_weak_diagonals_across_tiles(M):
     check(M, 20, np.random.default_rng(M))
 
 
-@pytest.mark.parametrize("M", [3073, 4100])
-def test_tile_rows_left_over_after_turns_of_eight(M):
-    """Every remainder of a tile's turns of eight rows, before and around a clearing row."""
-    check(M, 20, np.random.default_rng(8 * M), lengths=[*range(20), *range(112, 130)])
+@pytest.mark.parametrize("codes", [20, 25, 26])
+@pytest.mark.parametrize("M", [3073, 3840, 4096, 4100])
+def test_tile_rows_left_over_after_turns_of_eight(M, codes):
+    """Every remainder of a tile's turns of eight rows, before and around a
+    clearing row; tiles of 16 and 20 words (the latter hold 25 codes)."""
+    check(M, codes, np.random.default_rng(8 * M), lengths=[*range(20), *range(112, 130), 1201])
 
 
 LENGTHS = [3, 119, 120, 121, 122, 240, 243, 1201, 0, 1, 777, 2, 1802]
