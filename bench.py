@@ -43,12 +43,12 @@ OPS_PER_CELL = {"msv": 4, "ssv": 2}
 # ncu captures summarised in profiles/, keyed by kernel, workload and model
 # length; only used while the kernel is the one that was captured.
 NCU_TRAFFIC = {
-    # held MSV pass + its exact rescoring launch (profiles/scan_kernel_tmem_m2405_msweep500k.md)
-    ("scan_kernel<32,38,MSV_HELD,TMEM>", "msweep_500k", 2405): 187.900928e6 + 3.704576e6 + 0.258816e6,
-    ("scan_kernel<32,38,SSV,TMEM>", "msweep_500k", 2405): 187.970560e6 + 3.762432e6,
+    # held MSV pass + its exact rescoring launch (profiles/scan_kernel_row_pairs.md)
+    ("scan_kernel<32,38,MSV_HELD,TMEM>", "msweep_500k", 2405): 187.849728e6 + 3.647744e6 + 0.276224e6,
+    ("scan_kernel<32,38,SSV,TMEM>", "msweep_500k", 2405): 188.729856e6 + 0.141568e6,
 }
 KERNEL_SOURCE = os.path.join(ROOT, "paper_1707_09683_gb300", "csrc", "mpf_scan_kernel.cuh")
-KERNEL_SOURCE_SHA256 = "0e77766bf6a845c614e6a1de6f039389f88f67e468cac41aad9192c93c827c93"
+KERNEL_SOURCE_SHA256 = "82aca070535b127a2c0013d7298358c3b4f7a18b73b36f27fd2e6fa2e00821c2"
 
 
 def log(*a):
