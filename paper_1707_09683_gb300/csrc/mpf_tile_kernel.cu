@@ -336,19 +336,20 @@ __global__ void __launch_bounds__(kTileWarps * 32) tile_kernel(ScanParams sp) {
 // reads quarter w mod 4.  Warp w fills codes 8 (w / 4) .. + 7 of its quarter
 // from the tile in device memory.  One sequence per warp makes the residue
 // code of a row warp-uniform, so a row's P words are one or two tcgen05.ld
-// at one column address, issued
-// a row ahead into the other of two register buffers.
+// at one column address, issued a row ahead into the other of two register
+// buffers.
 //
 // The sweep keeps the largest cell V only, which decides MSV as in the striped
 // held pass: at or above 255 - bias - b some row overflowed, at most T the
 // held rows are exact, in between the sequence goes to the fallback list.
 // Rows go in pairs (16 ALU instructions for 16 words instead of 24).
 // Eight rows per loop turn, the words ahead in two registers each loaded in
-// place and lane 0's boundary word added instead of selected: a row has 24
-// instructions of cell work, and what surrounds it is what this saves.
-// Measured before / after, 20,000 sequences (M = 5,000: SSV 1.79 / 1.71 ms,
-// both filters 2.46 / 2.27; M = 3,500: SSV 1.43 / 1.37) and 5,000 (M =
-// 10,000: SSV 2.99 / 2.64).
+// place and lane 0's boundary word added instead of selected: a row of 16
+// words has 24 instructions of cell work, and what surrounds it is what this
+// saves.  Measured before / after with tiles of 16 words, 20,000 sequences
+// (M = 5,000: SSV 1.79 / 1.71 ms, both filters 2.46 / 2.27; M = 3,500: SSV
+// 1.43 / 1.37) and 5,000 (M = 10,000: SSV 2.99 / 2.64).  ncu, M = 5,000: 42
+// instructions per row, 24 of them on the ALU pipe, which is 81% busy.
 template <int P>
 __device__ __forceinline__ void tile_ld(uint32_t (&r)[P], uint32_t a) {
   static_assert(P == 16 || P == 20, "words per lane");
