@@ -76,7 +76,8 @@
 // segment, in order, and skips the segments whose largest cell is at most T:
 // with b constant over a segment no row of it can change xJ.  A segment
 // entered after a gap starts from a zero row seg_overlap <= seg_rows rows
-// earlier, in the skipped segment, over which b did not change either.
+// earlier, in the skipped segment, over which b did not change either.  One
+// that follows the segment before it goes on with the group's cells.
 //
 // The F16 modes hold the same integers as IEEE half values and update a cell
 // pair with one fused add-and-clamp-at-zero (HFMA2.RELU, v * 1 + s), which
@@ -610,13 +611,14 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
 
       // A rescored sequence that was split takes its segments one by one and
       // leaves out those whose largest cell cannot move xJ (see kUnits).
-      int seg = 0;
+      int seg = 0, left = 0;   // next segment, and words left of the current one
       bool follows = false;
       const int n_segs = kFast && active && r < p.n_long ? (int)(__ldg(p.unit_first + r + 1) - __ldg(p.unit_first + r)) : 1;
       for (;;) {
       if constexpr (kFast) {
-        busy = false;
-        if (active && !done) {
+        if (done) left = 0;
+        if (left == 0) busy = false;
+        if (left == 0 && active && !done) {
           while (n_segs > 1 && seg < n_segs && __ldcg(qd->unit_max + __ldg(p.unit_first + r) + seg) <= T) {
             ++seg;
             follows = false;
@@ -632,15 +634,21 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
 #pragma unroll
               for (int q = 0; q < H; ++q) v[q] = 0u;
             }
+            left = (rows + 3) >> 2;
             ++seg;
             follows = true;
           }
         }
         if (!__any_sync(kFull, busy)) break;
       }
-      nsteps = busy ? (rows + 3) >> 2 : 0;
+      nsteps = kFast ? left : busy ? (rows + 3) >> 2 : 0;
       wptr = busy ? wstart + ((uint32_t)first_row >> 2) : p.pad_word;
-      const int wsteps = (int)__reduce_max_sync(kFull, (uint32_t)nsteps);
+      int wsteps = (int)__reduce_max_sync(kFull, (uint32_t)nsteps);
+      // Past its segment's end a group would run padding rows, which clear the
+      // cells that its next segment follows on: the warp stops where the first
+      // such group ends, and the others go on with theirs in the next turn.
+      if constexpr (kFast && G > 1)
+        wsteps = min(wsteps, (int)__reduce_min_sync(kFull, busy && seg < n_segs ? (uint32_t)nsteps : (uint32_t)INT_MAX));
       cur = __ldg(p.residues + (nsteps > 0 ? wptr : p.pad_word));
       if constexpr (kUniform) cur = __reduce_max_sync(kFull, cur);
       ahead = __ldg(p.residues + (1 < nsteps ? wptr + 1u : p.pad_word));
@@ -703,6 +711,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
 
       if constexpr (TM) tm_wait_ld<HI>(thi);   // the load issued after the last row
       if constexpr (!kFast) break;
+      left = max(left - wsteps, 0);
+      first_row += 4 * wsteps;
+      rows -= 4 * wsteps;
       }
 
       // ---- finalise the G sequences -------------------------------------
