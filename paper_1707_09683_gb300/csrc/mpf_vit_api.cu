@@ -81,7 +81,8 @@ bool packable(mpf_vprofile *v, const int16_t *msc, const int16_t *trans) {
   v->pk_bm = tr(VT_BM, 0);
   const int floor = -32768 + kVitPackReach;
   const int lo = std::max(v->base + v->sp[1], -32768) + v->pk_bm - (v->pk_emax - 1);
-  return sink <= 1024 && v->pk_emax <= kVitPackReach && lo >= floor + 2048;
+  // A match state is at most the entry score plus pk_emax: it has to fit 16 bits.
+  return sink <= 1024 && v->pk_emax <= kVitPackReach && lo >= floor + 2048 && lo + v->pk_emax <= 32767;
 }
 
 // The packed tables of a shape, appended to *out; returns their offset.

@@ -42,8 +42,9 @@
 //     per profile): they sink at least as fast as the entry score.  At off =
 //     -kVitPackReach the floor is the true -32768 and nothing is conditional.
 //   * M is at most 32766 - off + (largest match score) before the row's
-//     overflow test: off starts at that score - 1, so M fits, and M >= 32767
-//     is seen exactly.  After off was lowered a row near the top of the range
+//     overflow test (the first entry score is at most 32766, checked per
+//     profile; a later one comes from a state of a row without overflow): off
+//     starts at that score - 1, so M fits, and M >= 32767 is seen exactly.  After off was lowered a row near the top of the range
 //     cannot be told from an overflow; such sequences, and rows whose best
 //     score is at the floor while it would matter, are left to the 32-bit
 //     kernels: their length ranks are appended to the query's list, which a

@@ -94,3 +94,22 @@ def test_profiles_at_the_edge_of_the_packed_form(kind):
         else:                              # no positive match score
             vp.msc = np.minimum(vp.msc, -1).astype(np.int16)
     check(vps, database(vps[1], rng, 4000))
+
+
+@pytest.mark.parametrize("top", [32767, 32766, 32765])
+@pytest.mark.parametrize("M", [2, 70, 600, 1400])
+def test_entry_score_at_the_top_of_the_range(M, top):
+    """A match state that overflows in the first row, beside others that stay
+    just below."""
+    rng = np.random.default_rng(M + top)
+    vp = synth.make_vit_profile(M, rng)
+    vp.base = top
+    vp.special[1] = 0
+    vp.trans[0] = 0
+    vp.msc[:] = -1
+    vp.msc[3:, rng.integers(0, M, 1 + M // 20)] = 5      # residue codes below 3: no overflow in their row
+    lengths = np.array([1, 1, 1, 2, 5, 40, 0, 300], dtype=np.uint32)
+    offsets = np.concatenate([[0], np.cumsum(lengths[:-1], dtype=np.uint64)]).astype(np.uint64)
+    res = rng.integers(0, 20, int(lengths.sum())).astype(np.uint8)
+    res[:3] = [0, 5, 19]
+    check([vp], synth.Database(residues=res, offsets=offsets, lengths=lengths))
