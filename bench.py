@@ -832,9 +832,18 @@ def run_batch_workload(args, ctx, idx, n_queries, time_steps, dev, steps=3):
     plans = {f: mpf.Plan(ctx, code, profs, db, *outs[f]) for f, code in filters}
     for pl in plans.values():
         pl.capture_graph()
-    narrow = [(pr, code) for pr in profs for _, code in filters if pr.get_config(code)[0] < 32]
-    for pr, code in narrow:
-        pr.set_table_memory(code, mpf.TABLE_SHARED)
+    # Queries that a plan may score several to a warp: fewer than 32 lanes once
+    # their table stays in shared memory (alone, some take the whole warp).
+    narrow = []
+    for pr, code in [(pr, code) for pr in profs for _, code in filters]:
+        tensor = pr.get_table_memory(code) == mpf.TABLE_TENSOR
+        if tensor:
+            pr.set_table_memory(code, mpf.TABLE_SHARED)
+        if pr.get_config(code)[0] < 32:
+            pr.set_table_memory(code, mpf.TABLE_SHARED)
+            narrow.append((pr, code))
+        elif tensor:
+            pr.set_table_memory(code, mpf.TABLE_AUTO)
     unpacked = {f: mpf.Plan(ctx, code, profs, db, *outs[f]) for f, code in filters}
     for pr, code in narrow:
         pr.set_table_memory(code, mpf.TABLE_AUTO)

@@ -140,9 +140,10 @@ void mpf_profile_destroy(mpf_profile *prof);
  * sequences per warp, W = 2 * lanes cells per row step, H = words).
  * set: MPF_EINVAL if the pair is not built or does not cover M, or if the
  *      profile is longer than mpf_max_striped_length() (one configuration).
- * get: writes the pair the next scan will use (tuned default if never set,
- *      where a scan may take a whole-warp kernel or a plan a mixed set instead:
- *      mpf_plan_group_info); lanes 32, words 0 for the long-model kernel.
+ * get: writes the pair the next scan of the query alone will use (tuned
+ *      default if never set); lanes 32, words 0 for the long-model kernel.  A
+ *      batch or plan of several queries may lay them out otherwise:
+ *      mpf_plan_group_info.
  */
 int mpf_profile_set_config(mpf_profile *prof, int filter, int lanes, int words);
 int mpf_profile_get_config(const mpf_profile *prof, int filter, int *lanes, int *words);
@@ -152,10 +153,13 @@ int mpf_profile_get_config(const mpf_profile *prof, int filter, int *lanes, int 
  * (for admission control by a server; not in the paper).  smem_bytes: the
  * shared memory one thread block of its kernel takes (the staged score table
  * or tile; for the lane-segment long-model kernel, one warp's DP row), with
- * the configuration the next scan will use.  table_bytes: the device memory
- * the profile's score tables for that kernel hold once built.  A scan also
- * writes 6 bytes per database sequence (raw, flag, nat) into the caller's
- * buffers.
+ * the configuration the next scan of the query alone will use.  table_bytes:
+ * the device memory the profile's score tables hold once built by that scan,
+ * those of its MSV rescoring launch included.  A batch or plan of several
+ * queries may lay them out otherwise and build more, which the profile keeps
+ * for later ones: per layout its table and, for MSV, those of its rescoring
+ * launches.  A scan also writes 6 bytes per database sequence (raw, flag, nat)
+ * into the caller's buffers.
  * Errors: MPF_EINVAL (null pointer or bad filter).
  */
 int mpf_profile_footprint(const mpf_profile *prof, int filter, uint32_t *smem_bytes,

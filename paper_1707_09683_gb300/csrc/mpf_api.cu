@@ -106,6 +106,20 @@ int alone_words(int M, int mode) {
   return w >= kTmMinWords && w <= kMaxWords && kernel_lg32_tm(w, mode) ? w : 0;
 }
 
+// (lanes, words) of a scan of this query alone with one filter: the pair that
+// was set, or the default.
+void scan_config(const mpf_profile *p, int filter, int mode, int *lanes, int *words) {
+  *lanes = p->cfg_lanes[filter];
+  *words = p->cfg_words[filter];
+  if (*lanes) return;
+  default_config(p->ctx, p->M, mode, lanes, words);
+  const int w = *lanes < 32 && p->table_mem[filter] != MPF_TABLE_SHARED ? alone_words(p->M, mode) : 0;
+  if (w) {
+    *lanes = 32;
+    *words = w;
+  }
+}
+
 // MSV_FAST needs the first begin score of every sequence below 255 - bias.
 bool msv_fast_ok(const mpf_profile *p) {
   int xb = p->base - (p->tjb_min + p->tbm);
@@ -850,18 +864,9 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       q.M = (uint32_t)p->M;
       q.seg_words = (uint32_t)p->seg_words;
     } else {
-      lanes = p->cfg_lanes[f];
-      words = p->cfg_words[f];
-      if (!lanes) {
-        default_config(ctx, p->M, mode, &lanes, &words);
-        // With others to share a warp with, that is decided below.
-        const int w = lanes < 32 && (n_q == 1 || ranks) && p->table_mem[f] != MPF_TABLE_SHARED
-                          ? alone_words(p->M, mode) : 0;
-        if (w) {
-          lanes = 32;
-          words = w;
-        }
-      }
+      scan_config(p, f, mode, &lanes, &words);
+      // With others to share a warp with, the whole warp is decided on below.
+      if (n_q > 1 && !ranks && !p->cfg_lanes[f]) default_config(ctx, p->M, mode, &lanes, &words);
       if (!lanes || !kernel_for(lanes, words, mode)) {
         plan_free(pl);
         return MPF_EUNSUPPORTED;
@@ -1582,8 +1587,8 @@ int mpf_profile_get_table_memory(const mpf_profile *p, int filter, int *where) {
                                                                                  : MPF_TABLE_SHARED;
     return MPF_OK;
   }
-  int lanes = p->cfg_lanes[filter], words = p->cfg_words[filter];
-  if (!lanes) default_config(p->ctx, p->M, mode, &lanes, &words);
+  int lanes = 0, words = 0;
+  scan_config(p, filter, mode, &lanes, &words);
   *where = use_tmem(p, filter, lanes, words, mode) ? MPF_TABLE_TENSOR : MPF_TABLE_SHARED;
   return MPF_OK;
 }
@@ -1593,11 +1598,8 @@ int mpf_profile_get_config(const mpf_profile *p, int filter, int *lanes, int *wo
   if (p->seg_words) {
     *lanes = 32;
     *words = 0;
-  } else if (p->cfg_lanes[filter]) {
-    *lanes = p->cfg_lanes[filter];
-    *words = p->cfg_words[filter];
   } else {
-    default_config(p->ctx, p->M, kernel_mode(p, filter), lanes, words);
+    scan_config(p, filter, kernel_mode(p, filter), lanes, words);
   }
   return MPF_OK;
 }
@@ -1620,12 +1622,20 @@ int mpf_profile_footprint(const mpf_profile *p, int filter, uint32_t *smem_bytes
     }
     return MPF_OK;
   }
-  int lanes = p->cfg_lanes[filter], words = p->cfg_words[filter];
-  if (!lanes) default_config(p->ctx, p->M, mode, &lanes, &words);
+  int lanes = 0, words = 0;
+  scan_config(p, filter, mode, &lanes, &words);
   if (!lanes) return MPF_EUNSUPPORTED;
   const TableGeom g = table_geom(lanes, words);
-  *smem_bytes = g.table_bytes;
+  // As configure_kernel: with the table in tensor memory, more than half.
+  *smem_bytes = use_tmem(p, filter, lanes, words, mode)
+                    ? std::max<uint32_t>(g.table_bytes, (uint32_t)p->ctx->max_smem / 2 + 1024)
+                    : g.table_bytes;
   *table_bytes = g.table_bytes;
+  // Rescoring launches after a held pass: the integer table beside an fp16
+  // one, and the table on 32 lanes beside a narrower one.
+  const bool held = mode == MODE_MSV_HELD || mode == MODE_MSV_HELD_F16;
+  if (mode == MODE_MSV_HELD_F16) *table_bytes += g.table_bytes;
+  if (held && lanes < 32) *table_bytes += table_geom(32, rescore_words(p->M)).table_bytes;
   return MPF_OK;
 }
 

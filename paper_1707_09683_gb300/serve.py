@@ -18,7 +18,8 @@ the work is drained:
 
 Footprint of a request (``Footprint``): the HBM it holds while in flight --
 its output slot (6 bytes per sequence and filter) and the device memory of
-its profile's score tables -- the shared memory one block of its kernels
+the score tables that its profile needs when scored alone (a batch that packs
+it with others may add some, about as large) -- the shared memory one block of its kernels
 takes (from the profile's kernel configuration), and its work, M x residues
 x 2 cells.  A request is admitted when its HBM bytes fit what the in-flight
 requests leave of ``hbm_budget`` and its work fits what they leave of
@@ -207,8 +208,10 @@ class ScanServer:
 
     def prepare(self, records):
         """Make these query profiles resident with their score tables built
-        (creating a plan builds them; nothing is launched), so the requests
-        that use them pay no set-up on the latency path."""
+        (creating a plan builds them; nothing is launched), so that a request
+        scored alone pays no set-up on the latency path.  The tables of a
+        layout that packs several queries into a warp are built by the first
+        batch that takes it."""
         sl = slice(0, 2 * self.n)
         for rec in records:
             prof = self._profile(rec)
