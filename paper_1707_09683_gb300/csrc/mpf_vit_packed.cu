@@ -575,20 +575,19 @@ int launch_viterbi_packed(const VitParams &p, VitPackShape s, int max_smem, int 
   const PackedFn fn = s.warps > 0 && s.warps <= kWarps ? packed_for(s) : nullptr;
   if (!fn) return 2;
   const int threads = s.warps > 1 ? 32 * s.warps : block_threads(s.qh, false);
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, (const void *)fn) != cudaSuccess) return 1;
   // A block with its transitions in tensor memory takes all of the SM's
-  // columns: it asks for more than half the shared memory, so that no second
-  // block that does so is placed on the SM.  The match scores come through
-  // the L1, which is left what the block (with under 8 KB of its own) does
-  // not use.
+  // columns: with its own shared memory it asks for more than half of what an
+  // SM has, so that no second block that does so is placed on the SM.  The
+  // match scores come through the L1, which is left the rest.
   const bool tm = in_tmem(s.qh, s.warps > 1);
-  const size_t smem = tm ? (size_t)max_smem / 2 + 1024 - 8192 : 0;
+  const size_t smem = tm ? (size_t)max_smem / 2 + 1024 - a.sharedSizeBytes : 0;
   int per_sm = 0;
   if (cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)fn, threads, smem) != cudaSuccess ||
       per_sm < 1 || (tm && per_sm != 1))
     return 1;
-  cudaFuncAttributes a;
-  if (cudaFuncGetAttributes(&a, (const void *)fn) != cudaSuccess) return 1;
   const int carve = (int)((size_t)per_sm * (smem + a.sharedSizeBytes + 1024) * 100 / (228 * 1024)) + 1;
   if (cudaFuncSetAttribute((const void *)fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve) != cudaSuccess)
     return 1;
