@@ -4,8 +4,8 @@
 // kernel_lg<MPF_LG>(): every mode of the striped scan kernel (eight) for each
 // built word count -- multiples of four, and the counts with a two-word tail.
 // With -DMPF_LG=32 -DMPF_TM=1 it builds kernel_lg32_tm() instead: the
-// tensor-memory variants (every mode but MSV_DIRECT, at least kTmMinWords
-// words).  With -DMPF_QP=1 (lanes 1 to 16) it builds kernel_qp_tm_lg<lanes>():
+// tensor-memory variants (SSV, held MSV and both in one sweep, at least
+// kTmMinWords words).  With -DMPF_QP=1 (lanes 1 to 16) it builds kernel_qp_tm_lg<lanes>():
 // the tensor-memory variants that score one sequence against 32 / lanes
 // queries per warp (integer SSV, the held MSV pass and the two together).
 // Either with -DMPF_FEW=1 builds the variants for databases of few residue
@@ -88,9 +88,7 @@ KernelFn kernel_lg32_tmfew(int words, int mode) {
 #define MPF_CASE(W)                                                                      \
   case W:                                                                                \
     if (mode == MODE_SSV) return scan_kernel<32, W, MODE_SSV, TM_ALL>;                   \
-    if (mode == MODE_MSV_FAST) return scan_kernel<32, W, MODE_MSV_FAST, TM_ALL>;         \
     if (mode == MODE_SSV_F16) return scan_kernel<32, W, MODE_SSV_F16, TM_ALL>;           \
-    if (mode == MODE_MSV_FAST_F16) return scan_kernel<32, W, MODE_MSV_FAST_F16, TM_ALL>; \
     if (mode == MODE_MSV_HELD) return scan_kernel<32, W, MODE_MSV_HELD, TM_ALL>;         \
     if (mode == MODE_MSV_HELD_F16) return scan_kernel<32, W, MODE_MSV_HELD_F16, TM_ALL>; \
     if (mode == MODE_MSV_SSV) return scan_kernel<32, W, MODE_MSV_SSV, TM_ALL>;           \

@@ -77,7 +77,6 @@ enum Mode : int {
                           //   gives both filters' scores
   MODE_TILE_MSV_SSV = 12, // MODE_TILE_MSV and MODE_TILE_SSV from one sweep (the same reason)
 };
-constexpr int kNumModes = 8;   // modes of the striped scan kernel
 
 // Striped kernels that read their table from tensor memory (one sequence per
 // warp): the first words of each lane's row of every residue code come from

@@ -192,7 +192,8 @@ __device__ __forceinline__ int mixed_max(int v, int lane, int gl, int width) {
 template <int LG, int H, int MODE, int TM = TM_NONE, int QP = 1, bool MIX = false>
 __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   static_assert((H % 4 == 0 || H % 4 == 2) && H >= 4 && H <= kMaxWords, "words per lane");
-  static_assert(!TM || ((LG == 32 || QP * LG == 32) && H >= kTmMinWords && MODE != MODE_MSV_DIRECT),
+  static_assert(!TM || ((LG == 32 || QP * LG == 32) && H >= kTmMinWords && MODE != MODE_MSV_DIRECT &&
+                        MODE != MODE_MSV_FAST && MODE != MODE_MSV_FAST_F16),
                 "tensor-memory variant");
   static_assert(QP == 1 || (TM && QP * LG == 32), "queries per warp");
   static_assert(!MIX || (TM == TM_FEW && LG == 32 && QP == 1 && tm_words(H, TM) == H), "mixed sets");
@@ -243,7 +244,6 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
   // Every lane of a warp follows the same sequence: a warp reduction (whose
   // result is uniform) hands each residue word to the rows.
   constexpr bool kUniform = TM != TM_NONE;
-  constexpr bool kTwoWords = kUniform && !kFast;
   constexpr bool kMapPad = TM == TM_FEW && HT == H;
   // Mixed sets: item i scores set i / n_shards, whose lanes belong to queries
   // as p.mix_lanes says (query, lane of its group, width; width 0: no query).
@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       }
 
       int since_clear = 0;
-      if constexpr (kTwoWords) {
+      if constexpr (kUniform) {
         // Two words per turn, loaded a turn ahead (unguarded: at most three
         // words past the rows, which lie in the database and are not scored).
         const uint32_t *wp = p.residues + wptr;
@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
       } else
       for (int step = 0; step < wsteps; ++step) {
         // Prefetch the residue words; past the end a group reads padding.
-        const uint32_t nxt = kUniform ? __reduce_max_sync(kFull, ahead) : ahead;
+        const uint32_t nxt = ahead;
         ahead = __ldg(p.residues + (step + 2 < nsteps ? wptr + (uint32_t)step + 2u : p.pad_word));
         if (kFast) {
           const bool near = busy && !done && (exact || Tnear < 0 || ((vacc + Tnear2) & 0x80008000u) != 0u);

@@ -47,7 +47,7 @@ __device__ __forceinline__ void tm_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// Loads of 16, 8, 4, 2 or 1 consecutive columns of the thread's lane into
+// Loads of 16, 8 or 4 consecutive columns of the thread's lane into
 // registers (32x32b shape).  The registers are valid only after tm_wait_ld.
 template <int N>
 __device__ __forceinline__ void tm_ld_pow2(uint32_t *r, uint32_t a);
@@ -75,14 +75,6 @@ __device__ __forceinline__ void tm_ld_pow2<4>(uint32_t *r, uint32_t a) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(a));
 }
-template <>
-__device__ __forceinline__ void tm_ld_pow2<2>(uint32_t *r, uint32_t a) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a));
-}
-template <>
-__device__ __forceinline__ void tm_ld_pow2<1>(uint32_t *r, uint32_t a) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[0]) : "r"(a));
-}
 
 // Eight or four columns starting OFF past column address a (as an immediate,
 // so that loads at one address share its uniform register).
@@ -97,18 +89,6 @@ __device__ __forceinline__ void tm_ld_at(uint32_t *r, uint32_t a) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4 + %5];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(a), "n"(OFF));
-}
-
-// N (< 32) consecutive columns starting at column address a.
-template <int N>
-__device__ __forceinline__ void tm_ld(uint32_t *r, uint32_t a) {
-  static_assert(N > 0 && N < 32, "columns per load");
-  constexpr int A = N & 16, B = N & 8, C = N & 4, D = N & 2, E = N & 1;
-  if constexpr (A) tm_ld_pow2<16>(r, a);
-  if constexpr (B) tm_ld_pow2<8>(r + A, a + A);
-  if constexpr (C) tm_ld_pow2<4>(r + A + B, a + A + B);
-  if constexpr (D) tm_ld_pow2<2>(r + A + B + C, a + A + B + C);
-  if constexpr (E) tm_ld_pow2<1>(r + A + B + C + D, a + A + B + C + D);
 }
 
 // Wait for this thread's outstanding tcgen05.ld; the empty asm statements
