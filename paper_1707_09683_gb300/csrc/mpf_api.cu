@@ -1657,7 +1657,7 @@ int mpf_db_upload(mpf_ctx *ctx, const uint8_t *residues, uint64_t n_residues,
     if (residues[i] >= 32) return MPF_EINVAL;
     seen |= 1u << residues[i];
   }
-  chunks += 1;  // the kernel prefetches one word past a sequence
+  chunks += 1;  // spare: the kernels read up to three words past a sequence's chunks
   if (chunks * 4 >= (1ull << 32)) return MPF_EUNSUPPORTED;
   // Length ranks: longest first, ties by sequence number.
   std::vector<uint32_t> order(n_seqs);

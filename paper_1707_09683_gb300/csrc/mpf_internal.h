@@ -70,7 +70,7 @@ enum Mode : int {
                           //   (with MODE_LONG_MSV over the sequences it leaves)
   MODE_MSV_HELD = 9,      // Alg. 2 with the begin score held for the whole sequence: no per-row
                           //   tests; sequences whose running maximum passes T are listed and
-                          //   rescored by MODE_MSV_DIRECT
+                          //   rescored by MODE_MSV_FAST
   MODE_MSV_HELD_F16 = 10, // MODE_MSV_HELD with cells as fp16 integers
   MODE_MSV_SSV = 11,      // MODE_MSV_HELD and MODE_SSV from one sweep: with b held the MSV
                           //   cells minus b follow the SSV recurrence, so the largest cell

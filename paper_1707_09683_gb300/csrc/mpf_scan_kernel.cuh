@@ -660,8 +660,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) scan_kernel(ScanParams p) {
 
       int since_clear = 0;
       if constexpr (kUniform) {
-        // Two words per turn, loaded a turn ahead (unguarded: at most three
-        // words past the rows, which lie in the database and are not scored).
+        // Two words per turn, loaded a turn ahead (unguarded: at most four
+        // words past the rows' last, three past its chunk; they lie in the
+        // database, whose last chunk is spare, and are not scored).
         const uint32_t *wp = p.residues + wptr;
         uint32_t a1 = ahead, a2 = __ldg(wp + 2);
         for (int step = 0; step < wsteps; step += 2) {
