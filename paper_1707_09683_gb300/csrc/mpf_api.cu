@@ -138,47 +138,60 @@ uint16_t half_bits(int v) {
   return (uint16_t)(sign | ((unsigned)(e + 15) << 10) | (m & 0x3ffu));
 }
 
+// Table entries by cost in the units of table format fmt (bias - cost), and at
+// 256 that of padding nodes and rows (kNegInf).
+struct TableEntries {
+  uint16_t at[257];
+  TableEntries(const mpf_profile *p, int fmt) {
+    const bool f16 = fmt == TABLE_F16;
+    for (int c = 0; c < 256; ++c)
+      at[c] = f16 ? half_bits(p->bias - c) : (uint16_t)(int16_t)((p->bias - c) * (1 << kCellShift));
+    at[256] = f16 ? half_bits(kNegInf) : (uint16_t)(int16_t)kNegInf;
+  }
+};
+
+// The entries of residue code x for nodes 0 .. n - 1 (n >= M).  Returns the
+// code's best score (kNegInf for the padding row).
+int table_row(const mpf_profile *p, const TableEntries &entry, int x, int n, uint16_t *row) {
+  const int M = p->M;
+  std::fill(row + (x < 32 ? M : 0), row + n, entry.at[256]);
+  if (x >= 32) return kNegInf;
+  if (x >= p->K) {
+    std::fill(row, row + M, entry.at[255]);
+    return p->bias - 255;
+  }
+  const uint8_t *cost = &p->cost[(size_t)x * M];
+  uint8_t low = 255;
+  for (int k = 0; k < M; ++k) {
+    row[k] = entry.at[cost[k]];
+    low = std::min(low, cost[k]);
+  }
+  return p->bias - low;
+}
+
 // Fill the striped shared-memory image of a profile for (lanes, words) in
 // table format fmt: 16-bit scores s = bias - cost per (copy, residue row,
-// word quad, lane, word, half), then 33 int16 per-code best scores.
+// word quad, lane, word, half), then 33 int16 per-code best scores.  The
+// first call on a profile waits for this.
 void fill_table_image(const mpf_profile *p, const TableGeom &g, int fmt, uint8_t *img) {
   memset(img, 0, g.table_bytes);
-  const int M = p->M, lanes = g.lanes, words = g.words;
-  // Signed score of node k (0-based) for residue code x; padding nodes and
-  // the padding code score kNegInf.
-  auto score = [&](int x, int k) -> int {
-    if (x >= 32 || k >= M) return kNegInf;
-    const int c = x < p->K ? (int)p->cost[(size_t)x * M + k] : 255;
-    return p->bias - c;
-  };
-  auto put = [&](size_t off, int x, int k) {
-    const int sv = score(x, k);
-    const uint16_t bits = fmt == TABLE_F16 ? half_bits(sv)
-                                           : (uint16_t)(int16_t)(sv == kNegInf ? kNegInf : sv * (1 << kCellShift));
-    memcpy(&img[off], &bits, 2);
-  };
-  const int qw = 4 * g.quads;   // words held in the quad region
-  for (int x = 0; x < kTableRows; ++x)
-    for (int l = 0; l < lanes; ++l)
-      for (int q = 0; q < words; ++q)
-        for (int h = 0; h < 2; ++h) {
-          const int k = (2 * l + h) * words + q;   // striped cell of (lane, half, word)
-          if (q < qw) {
-            for (int c = 0; c < g.copies; ++c)
-              put((size_t)c * g.copy_bytes + (size_t)x * g.row_bytes +
-                      ((size_t)(q / 4) * lanes + l) * 16 + (q % 4) * 4 + h * 2, x, k);
-          } else {
-            for (int c = 0; c < g.tail_copies; ++c)
-              put(g.tail_off + (size_t)x * g.tail_row_bytes + ((size_t)c * lanes + l) * 8 +
-                      (q - qw) * 4 + h * 2, x, k);
-          }
-        }
+  const int lanes = g.lanes, words = g.words, qw = 4 * g.quads;   // words held in the quad region
+  const TableEntries entry(p, fmt);
+  uint16_t row[2 * 32 * kMaxWords];
   for (int x = 0; x < kTableRows; ++x) {
-    int m = kNegInf;
-    if (x < 32)
-      for (int k = 0; k < M; ++k) m = std::max(m, score(x, k));
-    const int16_t sv = (int16_t)m;
-    memcpy(&img[g.smax_off + 2 * x], &sv, 2);
+    const int16_t best = (int16_t)table_row(p, entry, x, 2 * lanes * words, row);
+    memcpy(&img[g.smax_off + 2 * x], &best, 2);
+    uint8_t *quads = img + (size_t)x * g.row_bytes;
+    uint8_t *tail = img + g.tail_off + (size_t)x * g.tail_row_bytes;
+    for (int l = 0; l < lanes; ++l) {
+      const uint16_t *lo = row + 2 * l * words, *hi = lo + words;   // the striped cells of the lane's halves
+      for (int q = 0; q < words; ++q) {
+        const uint32_t w = lo[q] | (uint32_t)hi[q] << 16;
+        memcpy(q < qw ? quads + ((size_t)(q / 4) * lanes + l) * 16 + q % 4 * 4 : tail + (size_t)l * 8 + (q - qw) * 4, &w, 4);
+      }
+    }
+    for (int c = 1; c < g.copies; ++c) memcpy(quads + (size_t)c * g.copy_bytes, quads, (size_t)qw * lanes * 4);
+    for (int c = 1; c < g.tail_copies && g.tail_words; ++c) memcpy(tail + (size_t)c * lanes * 8, tail, (size_t)lanes * 8);
   }
 }
 
@@ -229,22 +242,15 @@ int get_mix_table(const mpf_profile *p, int lanes, int words, DevTable *out) {
   t.geom.smax_off = (uint32_t)(kTableRows * lanes * words * 4);
   t.geom.table_bytes = (t.geom.smax_off + 80u + 15u) & ~15u;
   std::vector<uint8_t> img(t.geom.table_bytes, 0);
-  int16_t *cell = reinterpret_cast<int16_t *>(img.data());
+  uint32_t *word = reinterpret_cast<uint32_t *>(img.data());
   int16_t *smax = reinterpret_cast<int16_t *>(&img[t.geom.smax_off]);
-  const int M = p->M;
+  const TableEntries entry(p, TABLE_I16);
+  uint16_t row[2 * 32 * kMaxWords];
   for (int x = 0; x < kTableRows; ++x) {
-    int m = kNegInf;
-    for (int k = 0; k < 2 * lanes * words; ++k) {
-      int s = kNegInf;
-      if (x < 32 && k < M) {
-        const int sv = p->bias - (x < p->K ? (int)p->cost[(size_t)x * M + k] : 255);
-        m = std::max(m, sv);
-        s = sv * (1 << kCellShift);
-      }
-      const int q = k % words, half = k / words % 2, l = k / words / 2;
-      cell[(((size_t)x * lanes + l) * words + q) * 2 + half] = (int16_t)s;
-    }
-    smax[x] = (int16_t)m;
+    smax[x] = (int16_t)table_row(p, entry, x, 2 * lanes * words, row);
+    for (int l = 0; l < lanes; ++l)
+      for (int q = 0; q < words; ++q)
+        *word++ = row[2 * l * words + q] | (uint32_t)row[(2 * l + 1) * words + q] << 16;
   }
   mpf_ctx *ctx = p->ctx;
   DeviceGuard dg(ctx->device);
@@ -829,6 +835,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     QueryDesc q;
     memset(&q, 0, sizeof(q));
     int lanes = 32, words = 0;
+    bool may_share = false;   // the warp with other queries (tables: once that is decided)
     if (mode == MODE_TILE_SSV || mode == MODE_TILE_MSV || mode == MODE_TILE_MSV_SSV) {
       const uint4 *tt = nullptr;
       const int ttm = tile_memory(p, f, db);
@@ -871,14 +878,16 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
         plan_free(pl);
         return MPF_EUNSUPPORTED;
       }
+      q.M = (uint32_t)p->M;
+      may_share = n_q >= 2 && !ranks && lanes < 32 && words >= kTmMinWords && p->table_mem[f] != MPF_TABLE_SHARED &&
+                  (mode == MODE_SSV || mode == MODE_MSV_HELD || mode == MODE_MSV_SSV);
       DevTable t;
-      int rc = get_table(p, lanes, words, table_format(mode), &t);
+      int rc = may_share ? MPF_OK : get_table(p, lanes, words, table_format(mode), &t);
       if (rc) {
         plan_free(pl);
         return rc;
       }
       set_table(q, t);
-      q.M = (uint32_t)p->M;
       if (mode == MODE_MSV_HELD || mode == MODE_MSV_HELD_F16 || mode == MODE_MSV_SSV) {
         // The integer table of the same layout, for the exact kernel that
         // rescores the sequences the held pass lists.
@@ -915,9 +924,7 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     const int tm = tiled ? tile_memory(p, f, db)
                          : p->seg_words ? 0 : (use_tmem(p, f, lanes, words, mode) ? 1 : 0);
     const int sf = p->seg_words ? 1 : p->shard_factor[f];
-    if (n_q >= 2 && !ranks && !p->seg_words && lanes < 32 &&
-        (mode == MODE_SSV || mode == MODE_MSV_HELD || mode == MODE_MSV_SSV) && words >= kTmMinWords &&
-        p->table_mem[f] != MPF_TABLE_SHARED) {
+    if (may_share) {
       int dl = 0, dw = 0;
       default_config(ctx, p->M, mode, &dl, &dw);
       qp_cand[std::make_pair(lanes, mode)].push_back(QpCand{words, sf, p, q, fb, p->cfg_lanes[f] == 0, lanes == dl && words == dw});
@@ -954,17 +961,16 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
       const GroupKey key0(lanes, H, mode, 1, QP);
       for (size_t j = a; j < b; ++j) {
         QueryDesc q = v[j].q;
-        DevTable fb = v[j].fb;
-        if (pack) {
-          DevTable t;
-          int rc = get_table(v[j].p, lanes, H, TABLE_I16_PACKED, &t);
-          if (rc == MPF_OK && mode != MODE_SSV) rc = get_table(v[j].p, lanes, H, TABLE_I16, &fb);
-          if (rc) {
-            plan_free(pl);
-            return rc;
-          }
-          set_table(q, t);
+        DevTable t, fb{};
+        int rc = MPF_OK;
+        if (!pack || mode != MODE_SSV) rc = get_table(v[j].p, lanes, H, TABLE_I16, &fb);
+        t = fb;
+        if (rc == MPF_OK && pack) rc = get_table(v[j].p, lanes, H, TABLE_I16_PACKED, &t);
+        if (rc) {
+          plan_free(pl);
+          return rc;
         }
+        set_table(q, t);
         const GroupKey key = pack ? key0 : GroupKey(lanes, v[j].words, mode, 0, 1);
         byconf[key].push_back(q);
         if (mode != MODE_SSV) fb_table[key].push_back(Rescore{fb, v[j].p});
@@ -1026,18 +1032,16 @@ int plan_create(mpf_ctx *ctx, int filter, const mpf_profile *const *profs, int n
     }
     for (size_t i = 0; i < v.size(); ++i) {
       if (placed[i]) continue;
-      const int w = mq[i].whole;
-      if (w) {
-        DevTable t;
-        const int rc = get_table(v[i].p, 32, w, TABLE_I16, &t);
-        if (rc) {
-          plan_free(pl);
-          return rc;
-        }
-        set_table(v[i].q, t);
-        v[i].fb = t;
+      const int w = mq[i].whole, lanes = w ? 32 : mq[i].lanes, words = w ? w : mq[i].words;
+      DevTable t;
+      const int rc = get_table(v[i].p, lanes, words, TABLE_I16, &t);
+      if (rc) {
+        plan_free(pl);
+        return rc;
       }
-      const GroupKey alone(w ? 32 : mq[i].lanes, w ? w : mq[i].words, mode, w ? 1 : 0, 1);
+      set_table(v[i].q, t);
+      v[i].fb = t;
+      const GroupKey alone(lanes, words, mode, w ? 1 : 0, 1);
       byconf[alone].push_back(v[i].q);
       if (mode != MODE_SSV) fb_table[alone].push_back(Rescore{v[i].fb, v[i].p});
       group_shards[alone] = std::max(group_shards[alone], v[i].sf);
