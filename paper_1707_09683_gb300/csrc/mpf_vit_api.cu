@@ -72,12 +72,16 @@ bool packable(mpf_vprofile *v, const int16_t *msc, const int16_t *trans) {
     }
   v->pk_emax = 1;
   v->pk_split = 0;
-  for (int x = 0; x < kVitRows; ++x)
-    for (int k = 0; k < M; ++k) {
-      const int s = x < K ? (int)msc[(size_t)x * M + k] : -32768;
-      v->pk_emax = std::max(v->pk_emax, s);
-      if (s < -kVitPackReach) v->pk_split |= 1u << x;
+  for (int x = 0; x < kVitRows; ++x) {
+    int low = x < K ? 0 : -32768, high = 0;
+    for (int k = 0; x < K && k < M; ++k) {
+      const int s = msc[(size_t)x * M + k];
+      low = std::min(low, s);
+      high = std::max(high, s);
     }
+    v->pk_emax = std::max(v->pk_emax, high);
+    if (low < -kVitPackReach) v->pk_split |= 1u << x;
+  }
   v->pk_bm = tr(VT_BM, 0);
   const int floor = -32768 + kVitPackReach;
   const int lo = std::max(v->base + v->sp[1], -32768) + v->pk_bm - (v->pk_emax - 1);
@@ -93,18 +97,30 @@ size_t append_packed(const mpf_vprofile *v, const int16_t *msc, const int16_t *t
   const size_t row = (size_t)words * 32, base = (out->size() + 127) & ~(size_t)127;
   out->resize(base + 2 * (kVitPackPlanes + 2 * (size_t)kVitRows) * row);
   int16_t *h = out->data() + base;   // half 0 is the low one
-  for (int k = 0; k < words * 64; ++k) {
-    const size_t seg = (size_t)k / QH, lane = seg / 2;    // lane over the team
-    const size_t at = 2 * (((lane / 32) * QH + k % QH) * 32 + lane % 32) + seg % 2;
-    for (int n = 0; n < kVitPackPlanes; ++n)
-      h[2 * (size_t)n * row + at] = k < M && !vit_move_unused(order[n], k, M) ? trans[(size_t)order[n] * M + k]
-                                                                               : (int16_t)-kVitPackReach;
-    for (int x = 0; x < kVitRows; ++x) {
-      const int sc = k >= M ? ((v->pk_split >> x) & 1u ? -32768 : -kVitPackReach)
-                     : x < K ? (int)msc[(size_t)x * M + k] : -32768;
-      const int first = std::max(sc, -kVitPackReach);
-      h[2 * (kVitPackPlanes + (size_t)x) * row + at] = (int16_t)first;
-      h[2 * (kVitPackPlanes + (size_t)kVitRows + x) * row + at] = (int16_t)(sc - first);
+  std::vector<uint32_t> at((size_t)M);   // each node's place in a row
+  for (int k = 0; k < M; ++k) {
+    const int seg = k / QH, lane = seg / 2;    // lane over the team
+    at[(size_t)k] = (uint32_t)(2 * ((lane / 32 * QH + k % QH) * 32 + lane % 32) + seg % 2);
+  }
+  // Plane by plane, filled with the value of the nodes past M; the second step
+  // of a code whose scores need none stays 0.
+  for (int n = 0; n < kVitPackPlanes; ++n) {
+    int16_t *d = h + 2 * (size_t)n * row;
+    std::fill(d, d + 2 * row, (int16_t)-kVitPackReach);
+    const int16_t *t = trans + (size_t)order[n] * M;
+    for (int k = 0; k < M; ++k)
+      if (!vit_move_unused(order[n], k, M)) d[at[(size_t)k]] = t[k];
+  }
+  for (int x = 0; x < kVitRows; ++x) {
+    int16_t *d = h + 2 * (kVitPackPlanes + (size_t)x) * row, *d2 = d + 2 * kVitRows * row;
+    std::fill(d, d + 2 * row, (int16_t)-kVitPackReach);
+    const int16_t *sc = msc + (size_t)x * M;
+    const bool split = (v->pk_split >> x) & 1u;
+    if (split) std::fill(d2, d2 + 2 * row, (int16_t)(-32768 + kVitPackReach));
+    for (int k = 0; x < K && k < M; ++k) {
+      const int first = std::max((int)sc[k], -kVitPackReach);
+      d[at[(size_t)k]] = (int16_t)first;
+      if (split) d2[at[(size_t)k]] = (int16_t)(sc[k] - first);
     }
   }
   return base;
@@ -442,6 +458,10 @@ int mpf_vit_profile_create(mpf_ctx *ctx, int M, int K, const int16_t *msc, const
   // One allocation and one copy: match scores, transitions, packed tables.
   v->packed = packable(v, msc, trans);
   const size_t hm_n = hm.size();
+  size_t total = hm.size() + ht.size();
+  for (const VitPackShape &s : {v->pack_solo, v->pack_team})
+    total += v->packed ? 128 + 2 * (kVitPackPlanes + 2 * (size_t)kVitRows) * (size_t)(s.warps * s.qh) * 32 : 0;
+  hm.reserve(total);
   hm.insert(hm.end(), ht.begin(), ht.end());
   size_t solo = 0, team = 0;
   if (v->packed && v->pack_solo.warps) solo = append_packed(v, msc, trans, v->pack_solo, &hm);
