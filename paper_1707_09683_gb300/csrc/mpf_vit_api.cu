@@ -204,6 +204,7 @@ int64_t pack_team_max(const mpf_vprofile *v, int num_sms) {
 // shape).  *buf: a stream-ordered allocation that the caller frees after the
 // launches that read the lists of sequences left to the 32-bit kernels:
 // query i's list at fb_ranks[i], its count at fb_count[i] (null: not packed).
+// MPF_ENOMEM: nothing was launched and both are null throughout.
 int packed_enqueue(mpf_ctx *ctx, const mpf_vprofile *const *vps, int n_q, const mpf_db *db, int16_t *score,
                    uint8_t *flag, float *nat, const uint32_t *ranks, const uint32_t *n_ranks, uint8_t **buf,
                    std::vector<uint32_t *> *fb_ranks, std::vector<uint32_t *> *fb_count) {
@@ -401,6 +402,8 @@ int viterbi_enqueue(mpf_ctx *ctx, const mpf_vprofile *const *vps, int n_q, const
   uint8_t *buf = nullptr;
   std::vector<uint32_t *> fb_ranks, fb_count;
   int rc = packed_enqueue(ctx, vps, n_q, db, score, flag, nat, ranks, n_ranks, &buf, &fb_ranks, &fb_count);
+  // No room for the lists: the 32-bit kernels, which need none, score them all.
+  if (rc == MPF_ENOMEM) rc = MPF_OK;
   if (rc == MPF_OK) {
     std::vector<const uint32_t *> rk((size_t)n_q), nr((size_t)n_q);
     for (size_t q = 0; q < (size_t)n_q; ++q) {
