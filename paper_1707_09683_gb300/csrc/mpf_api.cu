@@ -97,8 +97,10 @@ void default_config(const mpf_ctx *ctx, int M, int mode, int *lanes, int *words)
 // default configuration when it is alone in a warp, or 0.  Above kAloneTmM
 // nodes the tensor-memory kernel is ahead of the narrow groups, whose rows
 // are bound by shared-memory reads (SSV, 60,000 sequences, ms narrow / whole
-// warp: M = 448 0.56 / 0.54, 512 0.64 / 0.54, 640 0.81 / 0.65, 800 0.98 / 0.79,
-// 1,024 1.28 / 0.91).
+// warp: M = 449 0.58 / 0.56, 512 0.62 / 0.56, 640 0.77 / 0.62, 800 0.99 / 0.77,
+// 1,024 1.20 / 0.88, 1,280 1.48 / 1.03; with a residue code of 20 or more, which
+// leaves 12 words per lane in tensor memory from 16 on, 1,024 1.20 / 0.89, 1,280
+// 1.48 / 1.09).
 constexpr int kAloneTmM = 448;
 int alone_words(int M, int mode) {
   if (M <= kAloneTmM || (mode != MODE_SSV && mode != MODE_MSV_HELD && mode != MODE_MSV_SSV)) return 0;

@@ -11,9 +11,10 @@
 // scores (one 32-bit word per two nodes, L1) and nothing of its own.  What
 // bounds it: the ALU pipe, 77-85% busy at M = 400-2405 (a DPX instruction
 // takes two cycles per warp and scheduler); launches with few sequences are
-// bound by a row's chain of dependent steps.  Measured (GB300, one query, ms,
-// the 32-bit kernels before / now): M = 400 on 20,000 sequences 4.37 / 1.55,
-// M = 2405 26.3 / 6.84 (2,470 GCUPS), M = 150 on 1,000 1.68 / 0.76.
+// bound by a row's chain of dependent steps.  Measured (GB300, one query, calls
+// back to back, random sequences of mean 355, ms, the 32-bit kernels before /
+// now): M = 400 on 20,000 sequences 4.47 / 1.70, M = 2405 27.4 / 6.89 (2,457
+// GCUPS), M = 150 on 1,003 1.68 / 0.68.
 //
 // Layout.  A warp, or a team of W warps, scores one sequence.  In node order
 // the team's warps, their lanes and the two halves of a lane's words form one chain of
