@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(block_threads(QH, TEAM), block_min(QH, TEAM))
       if (!MPF_DCHECK(p.status, r < p.n_seqs)) continue;
       const uint32_t w0 = __ldg(p.seq_word + r);
       const int len = (int)__ldg(p.seq_len + r);
-      if (!MPF_DCHECK(p.status, (uint64_t)w0 + (uint64_t)((len + 3) >> 2) + 1 <= p.n_words)) continue;
+      if (!MPF_DCHECK(p.status, (uint64_t)w0 + (uint64_t)((len + 3) >> 2) + 2 <= p.n_words)) continue;
 
       // Short lanes load a row's match scores while the row before ends, long
       // ones a few words ahead.
